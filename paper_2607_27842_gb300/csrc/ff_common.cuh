@@ -455,8 +455,8 @@ cudaError_t launch_noise(unsigned long long seed, float* out, long long n, cudaS
 cudaError_t launch_pos2d(DType dt, void* out, int B, int gh, int gw, int C, cudaStream_t s);
 
 // dense layers: out = epilogue(A[M,K] W[N,K]^T)
-cudaError_t gemm_simt(DType dt, int M, int N, int K, const void* A, int lda, const void* W, int ldw,
-                      const EpiArgs& e, cudaStream_t s);
+cudaError_t gemm_f32(int M, int N, int K, const float* A, int lda, const float* W, int ldw, const EpiArgs& e,
+                     cudaStream_t s);
 cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, int ldw, const EpiArgs& e,
                     cudaStream_t s);
 // Two problems of the same N and K (A0 W0^T with epilogue e0 over M0 rows and

@@ -84,7 +84,7 @@ featfix_status featfix_op_gemm(int dtype, int M, int N, int K, const void* dev_a
   e.hist_base = dev_hist_base;
   e.hist_out = dev_hist_out;
   if (dtype == FEATFIX_DTYPE_BF16) return st(gemm_tc(M, N, K, dev_a, K, dev_w, K, e, (cudaStream_t)stream));
-  return st(gemm_simt(F32, M, N, K, dev_a, K, dev_w, K, e, (cudaStream_t)stream));
+  return st(gemm_f32(M, N, K, (const float*)dev_a, K, (const float*)dev_w, K, e, (cudaStream_t)stream));
 }
 
 featfix_status featfix_op_attention(int dtype, const void* dev_qkv, int ld_qkv, void* dev_out, int ld_out, int batch,

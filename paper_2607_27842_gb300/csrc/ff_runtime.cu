@@ -440,7 +440,7 @@ const void* coff(const void* base, long long elems, int es) { return reinterpret
 cudaError_t dense(featfix_ctx* c, int M, int N, int K, const void* A, int lda, const void* W, const EpiArgs& e) {
   KTimer tm(c, FEATFIX_KCLASS_GEMM, 2.0 * M * N * (double)K);
   if (c->dt == BF16) return gemm_tc(M, N, K, A, lda, W, K, e, c->st);
-  return gemm_simt(c->dt, M, N, K, A, lda, W, K, e, c->st);
+  return gemm_f32(M, N, K, (const float*)A, lda, (const float*)W, K, e, c->st);
 }
 
 // Two streams' layers of the same shape (image rows M0, text rows M1) in one

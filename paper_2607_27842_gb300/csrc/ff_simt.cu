@@ -2,78 +2,289 @@
 // mode of the exact block (Eq. 1) and the narrow final projection.
 #include "ff_common.cuh"
 
+#include <cooperative_groups.h>
 #include <math.h>
+
+#include <algorithm>
+#include <type_traits>
+
+namespace cg = cooperative_groups;
 
 namespace ff {
 
-// ---------------------------------------------------------------------------
-// out = epilogue(A[M,K] W[N,K]^T), 64 x 128 tile, BK = 16, each thread owns
-// 4 rows x 8 consecutive columns.  Operands are converted to fp32 in shared
-// memory; accumulation is fp32 FFMA.
-// ---------------------------------------------------------------------------
-constexpr int SG_BM = 64, SG_BN = 128, SG_BK = 16;
-
-template <class T>
-__global__ void __launch_bounds__(256) k_gemm_simt(int M, int N, int K, const T* __restrict__ A, int lda,
-                                                   const T* __restrict__ W, int ldw, EpiArgs e) {
-  __shared__ __align__(16) float As[SG_BK][SG_BM + 4];
-  __shared__ __align__(16) float Ws[SG_BK][SG_BN + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * SG_BM, n0 = blockIdx.x * SG_BN;
-  float acc[4][8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-
-  for (int k0 = 0; k0 < K; k0 += SG_BK) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int idx = threadIdx.x + q * 256;  // 0 .. 1023 over [64 rows][16 k]
-      const int r = idx >> 4, kk = idx & 15;
-      const int gm = m0 + r, gk = k0 + kk;
-      As[kk][r] = (gm < M && gk < K) ? to_f(A[(size_t)gm * lda + gk]) : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int idx = threadIdx.x + q * 256;  // 0 .. 2047 over [128 rows][16 k]
-      const int r = idx >> 4, kk = idx & 15;
-      const int gn = n0 + r, gk = k0 + kk;
-      Ws[kk][r] = (gn < N && gk < K) ? to_f(W[(size_t)gn * ldw + gk]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < SG_BK; ++kk) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Ws[kk][tx * 8]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Ws[kk][tx * 8 + 4]);
-      const float a[4] = {a4.x, a4.y, a4.z, a4.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  const int nc = n0 + tx * 8;
-  if (nc >= N) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m < M) epi_chunk<T, 8>(e, m, nc, N, acc[i]);
-  }
+static int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 148;
+  }();
+  return n;
 }
 
-cudaError_t gemm_simt(DType dt, int M, int N, int K, const void* A, int lda, const void* W, int ldw,
-                      const EpiArgs& e, cudaStream_t s) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  dim3 grid((N + SG_BN - 1) / SG_BN, (M + SG_BM - 1) / SG_BM);
-  if (dt == F32)
-    k_gemm_simt<float><<<grid, 256, 0, s>>>(M, N, K, (const float*)A, lda, (const float*)W, ldw, e);
-  else
-    k_gemm_simt<bf16><<<grid, 256, 0, s>>>(M, N, K, (const bf16*)A, lda, (const bf16*)W, ldw, e);
+// ---------------------------------------------------------------------------
+// out = epilogue(A[M,K] W[N,K]^T) in fp32 on CUDA cores, FFMA2.
+//
+// Both operands are K-contiguous, so their tiles are copied to shared memory
+// as they are (cp.async, ST stages of BK columns, rows padded by 16 bytes:
+// eight consecutive rows' 16-byte vectors fall into distinct banks), and a
+// thread's TM x TN outputs accumulate (even k, odd k) pairs with fma.rn.f32x2:
+// the 16-byte fragment loads need no transposition and no duplicated operand,
+// and each output is two interleaved partial sums.  WK groups of warps share a
+// tile, each taking its own 16-byte columns of every stage; the groups'
+// accumulators are added through shared memory in a fixed order.  Several
+// CTAs of a cluster may share a tile's K range as well (small problems, where
+// the tiles alone leave the chip idle and the serial loads are the time);
+// they add through distributed shared memory, rank by rank, so the result
+// does not depend on timing.
+//
+// Bound: FFMA2 issue beside the fragment loads.  A register-only FFMA2 loop
+// runs at 114 of the 128 FMA per SM and clock (scalar FFMA 76), with this
+// kernel's 16 16-byte loads per 256 FMA 91; the 128 tile reaches 83.  What
+// counted: deep stages (BK 32 -> 128 on 64 tiles: 512 x 1152 x 1152 42 -> 36
+// us; every barrier leaves all warps waiting on their first loads) and copies
+// whose addresses cost one addition (1024 x 4608 x 4608 985 -> 870 us, 50
+// TFLOP/s).  Against 4-byte staging loads, one buffer and 64 x 128 tiles
+// everywhere: the 4-block fp32 sampling run 2952 -> 832 us, a DiT-XL/2 block
+// of 512 rows (attention included) 2235 -> 1049 us.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool in) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp4(void* dst, const void* src, bool in) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void ffma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+// BM x BN tile, warp tile 8 TM x 4 TN (lanes 8 x 4), WK groups of warps
+template <int BM_, int BN_, int TM_, int TN_, int WK_, int BK_, int ST_> struct F32Cfg {
+  static constexpr int BM = BM_, BN = BN_, TM = TM_, TN = TN_, WK = WK_, BK = BK_, ST = ST_;
+  static constexpr int WM = 8 * TM, WN = 4 * TN;
+  static constexpr int WARPS_M = BM / WM, WARPS_N = BN / WN;
+  static constexpr int THREADS = 32 * WARPS_M * WARPS_N * WK;
+  static constexpr int LD = BK + 4;                    // row stride of a staged operand (floats)
+  static constexpr int STAGE = (BM + BN) * LD;         // floats of a stage
+  static constexpr int LDC = BN + 4;                   // row stride of an output tile
+  static constexpr int RED = WK * BM * LDC;            // the groups' output tiles, over the stages
+  static constexpr size_t SMEM = sizeof(float) * (size_t)(ST * STAGE > RED ? ST * STAGE : RED);
+  static_assert((BK / 4) % WK == 0, "every group takes whole 16-byte columns");
+};
+
+template <class C, bool VEC>
+__global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, const float* __restrict__ A, int lda,
+                                                         const float* __restrict__ W, int ldw,
+                                                         const __grid_constant__ EpiArgs e) {
+  extern __shared__ __align__(16) float sm[];
+  pdl_trigger();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wk = warp / (C::WARPS_M * C::WARPS_N), wt = warp % (C::WARPS_M * C::WARPS_N);
+  const int lm = lane >> 2, ln = lane & 3;
+  const int ra = (wt / C::WARPS_N) * C::WM + lm;       // the thread's A rows: ra + 8 i
+  const int rb = (wt % C::WARPS_N) * C::WN + ln;       // its W rows: rb + 4 j
+  // one-dimensional grid over the tiles, row blocks fastest: the CTAs running
+  // together share W tiles (rows are few, W is the larger operand)
+  const int num_m = (M + C::BM - 1) / C::BM;
+  const int m0 = (int)(blockIdx.x % num_m) * C::BM, n0 = (int)(blockIdx.x / num_m) * C::BN;
+  const int split = gridDim.y, rank = blockIdx.y;
+  const int nkt = (K + C::BK - 1) / C::BK;
+  const int kt0 = (int)((long long)nkt * rank / split), kt1 = (int)((long long)nkt * (rank + 1) / split);
+
+  // Copies: the thread's column of a stage and its rows (r0 + RPP q of A, then
+  // of W) are fixed, so a copy costs one address addition; rows past the end
+  // and columns past K are zeros that read nothing.
+  constexpr int EL = VEC ? 4 : 1, CPR = C::BK / EL, RPP = C::THREADS / CPR;
+  constexpr int PA = C::BM / RPP, PW = C::BN / RPP;
+  static_assert(C::BM % RPP == 0 && C::BN % RPP == 0 && PA + PW <= 64, "whole passes");
+  using Mask = typename std::conditional<PA + PW <= 32, unsigned, unsigned long long>::type;
+  // row offsets from the tile's first row (32 bits on the 16-byte path, whose
+  // row strides the dispatch bounds)
+  using Off = typename std::conditional<VEC, unsigned, size_t>::type;
+  const int kc = (tid % CPR) * EL, r0 = tid / CPR;
+  const Off oa = (Off)r0 * (Off)lda + kc, ow = (Off)r0 * (Off)ldw + kc;
+  Mask live = 0;                                   // bit q: row r0 + RPP q of A, bit PA + q: of W
+#pragma unroll
+  for (int q = 0; q < PA; ++q) live |= (Mask)(m0 + r0 + RPP * q < M ? 1 : 0) << q;
+#pragma unroll
+  for (int q = 0; q < PW; ++q) live |= (Mask)(n0 + r0 + RPP * q < N ? 1 : 0) << (PA + q);
+  const float* const At = A + (size_t)m0 * lda;
+  const float* const Wt = W + (size_t)n0 * ldw;
+  auto load = [&](int kt, int slot) {
+    float* s = sm + slot * C::STAGE + r0 * C::LD + kc;
+    const int k0 = kt * C::BK;
+    const Mask mask = k0 + kc < K ? live : (Mask)0;
+#pragma unroll
+    for (int q = 0; q < PA + PW; ++q) {
+      const bool in = (mask >> q) & 1;
+      const float* src = q < PA ? At + k0 + (oa + (Off)(RPP * q) * (Off)lda)
+                                : Wt + k0 + (ow + (Off)(RPP * (q - PA)) * (Off)ldw);
+      src = in ? src : A;
+      float* d = s + (q < PA ? RPP * q : C::BM + RPP * (q - PA)) * C::LD;
+      if (VEC) cp16(d, src, in); else cp4(d, src, in);
+    }
+  };
+
+  unsigned long long acc[C::TM][C::TN];
+#pragma unroll
+  for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+    for (int j = 0; j < C::TN; ++j) acc[i][j] = 0ull;
+
+  pdl_wait();
+#pragma unroll
+  for (int p = 0; p < C::ST - 1; ++p) {
+    if (kt0 + p < kt1) load(kt0 + p, p);
+    cp_commit();
+  }
+  for (int kt = kt0; kt < kt1; ++kt) {
+    cp_wait<C::ST - 2>();
+    __syncthreads();
+    const int it = kt - kt0;
+    if (kt + C::ST - 1 < kt1) load(kt + C::ST - 1, (it + C::ST - 1) % C::ST);
+    cp_commit();
+    const float* sa = sm + (it % C::ST) * C::STAGE + ra * C::LD;
+    const float* sb = sm + (it % C::ST) * C::STAGE + (C::BM + rb) * C::LD;
+#pragma unroll
+    for (int c = 0; c < C::BK / 4 / C::WK; ++c) {
+      const int kk = (c * C::WK + wk) * 4;
+      ulonglong2 a[C::TM], b[C::TN];
+#pragma unroll
+      for (int i = 0; i < C::TM; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(sa + 8 * i * C::LD + kk);
+#pragma unroll
+      for (int j = 0; j < C::TN; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(sb + 4 * j * C::LD + kk);
+#pragma unroll
+      for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+        for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].x, b[j].x);
+#pragma unroll
+      for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+        for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].y, b[j].y);
+    }
+  }
+  cp_wait<0>();
+  __syncthreads();                                     // the stages are free: output tiles over them
+  {
+    float* t = sm + wk * C::BM * C::LDC;
+#pragma unroll
+    for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+      for (int j = 0; j < C::TN; ++j)
+        t[(ra + 8 * i) * C::LDC + rb + 4 * j] =
+            __uint_as_float((unsigned)acc[i][j]) + __uint_as_float((unsigned)(acc[i][j] >> 32));
+  }
+  __syncthreads();
+  // four consecutive columns of one row per thread: the groups' partials in
+  // order, then (split) the ranks' tiles in order, then the epilogue
+  constexpr int CPT = C::BN / 4;
+  auto group_sum = [&](int r, int c4) {
+    float4 v = *reinterpret_cast<const float4*>(sm + r * C::LDC + 4 * c4);
+#pragma unroll
+    for (int g = 1; g < C::WK; ++g) {
+      const float4 u = *reinterpret_cast<const float4*>(sm + (g * C::BM + r) * C::LDC + 4 * c4);
+      v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+    }
+    return v;
+  };
+  auto finish = [&](int r, int c4, const float4& v) {
+    const int m = m0 + r, n = n0 + 4 * c4;
+    if (m >= M || n >= N) return;
+    float x[4] = {v.x, v.y, v.z, v.w};
+    epi_chunk<float, 4, 0>(e, m, n, N, x);
+  };
+  if (split == 1) {
+    for (int c = tid; c < C::BM * CPT; c += C::THREADS) finish(c / CPT, c % CPT, group_sum(c / CPT, c % CPT));
+    return;
+  }
+  for (int c = tid; C::WK > 1 && c < C::BM * CPT; c += C::THREADS)
+    *reinterpret_cast<float4*>(sm + (c / CPT) * C::LDC + 4 * (c % CPT)) = group_sum(c / CPT, c % CPT);
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();
+  const int rows = C::BM / split;                      // this rank finishes rows [rank * rows, + rows)
+  for (int c = tid; c < rows * CPT; c += C::THREADS) {
+    const int r = rank * rows + c / CPT, c4 = c % CPT;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < split; ++q) {
+      const float4 u = *reinterpret_cast<const float4*>(cluster.map_shared_rank(sm, q) + r * C::LDC + 4 * c4);
+      v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+    }
+    finish(r, c4, v);
+  }
+  cluster.sync();                                      // peers may still be reading this CTA's tile
+}
+
+template <class C, bool VEC>
+static cudaError_t gemm_f32_launch(int M, int N, int K, const float* A, int lda, const float* W, int ldw,
+                                   const EpiArgs& e, int split, cudaStream_t s) {
+  const cudaError_t attr =
+      cudaFuncSetAttribute(k_gemm_f32<C, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  if (attr != cudaSuccess) return attr;
+  const long long tiles = (long long)((N + C::BN - 1) / C::BN) * ((M + C::BM - 1) / C::BM);
+  if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)tiles, split);
+  cfg.blockDim = dim3(C::THREADS);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 1;
+  at[1].val.clusterDim.y = split;
+  at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = split > 1 ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, k_gemm_f32<C, VEC>, M, N, K, A, lda, W, ldw, e);
   return launched();
+}
+
+// Tile choice by the estimated time of the launch's waves (one 128 or 64 tile
+// per SM at a time; a 64 tile's FMA count at 0.9 of the 128 tile's rate, a 32
+// tile's at 0.6).  Few rows or few tiles are latency- or weight-bound: 16 x 32
+// tiles up to 16 rows (W read once per 16 rows: 2 x 6912 x 1152 22.7 -> 15.2
+// us) and wherever 32 x 32 tiles would leave half the SMs idle (64 x 512 x 128
+// 3.46 -> 2.86 us); those also split K over a cluster while every CTA keeps a
+// K range of at least 128 (a split costs about 1 us: 64 x 128 x 128 in two
+// halves 3.46 -> 3.98 us).
+template <bool VEC>
+static cudaError_t gemm_f32_t(int M, int N, int K, const float* A, int lda, const float* W, int ldw, const EpiArgs& e,
+                              cudaStream_t s) {
+  using C128 = F32Cfg<128, 128, 8, 8, 1, 64, 3>;
+  using C64 = F32Cfg<64, 64, 8, 8, 4, 128, 2>;
+  using C32 = F32Cfg<32, 32, 4, 8, 8, 64, 4>;
+  using C16 = F32Cfg<16, 32, 2, 8, 8, 128, 3>;
+  const long long sms = sm_count();
+  const long long t128 = (long long)((M + 127) / 128) * ((N + 127) / 128);
+  const long long t64 = (long long)((M + 63) / 64) * ((N + 63) / 64);
+  const long long t32 = (long long)((M + 31) / 32) * ((N + 31) / 32);
+  if (M > 16 && t32 * 2 > sms) {
+    const double c128 = (double)((t128 + sms - 1) / sms) * 128 * 128;
+    const double c64 = (double)((t64 + sms - 1) / sms) * 64 * 64 * 1.1;
+    const double c32 = std::max(1.0, (double)t32 / sms) * 32 * 32 * 1.6;
+    if (c128 <= c64 && c128 <= c32) return gemm_f32_launch<C128, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
+    if (c64 <= c32) return gemm_f32_launch<C64, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
+    return gemm_f32_launch<C32, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
+  }
+  const long long t16 = (long long)((M + 15) / 16) * ((N + 31) / 32);
+  int split = 1;
+  while (split < 8 && t16 * split * 2 <= 2 * sms && K / (split * 2) >= 128) split *= 2;
+  return gemm_f32_launch<C16, VEC>(M, N, K, A, lda, W, ldw, e, split, s);
+}
+
+cudaError_t gemm_f32(int M, int N, int K, const float* A, int lda, const float* W, int ldw, const EpiArgs& e,
+                     cudaStream_t s) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  const bool vec = K % 4 == 0 && lda % 4 == 0 && ldw % 4 == 0 && !((uintptr_t)A & 15) && !((uintptr_t)W & 15) &&
+                   lda <= (1 << 24) && ldw <= (1 << 24);
+  return vec ? gemm_f32_t<true>(M, N, K, A, lda, W, ldw, e, s) : gemm_f32_t<false>(M, N, K, A, lda, W, ldw, e, s);
 }
 
 // ---------------------------------------------------------------------------
