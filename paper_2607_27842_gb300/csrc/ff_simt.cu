@@ -45,8 +45,8 @@ static int sm_count() {
 // us; every barrier leaves all warps waiting on their first loads) and copies
 // whose addresses cost one addition (1024 x 4608 x 4608 985 -> 870 us, 50
 // TFLOP/s).  Against 4-byte staging loads, one buffer and 64 x 128 tiles
-// everywhere: the 4-block fp32 sampling run 2952 -> 832 us, a DiT-XL/2 block
-// of 512 rows (attention included) 2235 -> 1049 us.
+// everywhere: 1024 x 4608 x 4608 1775 -> 870 us, 512 x 1152 x 4608 562 -> 131,
+// 64 x 128 x 512 60 -> 4.3, 2 x 6912 x 1152 122 -> 15.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp16(void* dst, const void* src, bool in) {
   const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -288,78 +288,203 @@ cudaError_t gemm_f32(int M, int N, int K, const float* A, int lda, const float* 
 }
 
 // ---------------------------------------------------------------------------
-// Attention on CUDA cores: one warp per query row, keys in chunks of 32
-// (lane j scores key j of the chunk), online softmax, each lane owns output
-// dims lane, lane + 32, ... (d <= 128).
+// Attention on CUDA cores in fp32 (fp32 mode, and bf16 head widths without a
+// tensor-core kernel): one CTA per (sample, head, 32 queries), 64 keys at a
+// time through shared memory, 128 threads as 8 query groups x 16 lanes.
+// Thread (tq, tk) owns queries tq + 8 i (i < 4): their scores against keys
+// tk + 16 j, then, after the online softmax over the group's 16 lanes, output
+// columns 2 tk + 32 g of the same queries (DG column pairs per lane).  P goes
+// through shared memory but stays within its group of lanes.  The next tile's
+// keys are copied while the softmax and P V run, its values while the next
+// scores are computed (cp.async into the one buffer each).
+//
+// Bound: shared-memory fragment loads (8 per 64 FMA in q k^T, 16 per 96 in
+// P V at head width 72).  Against one warp per query reading keys row by row
+// from global memory (uncoalesced, no reuse): 2 x 256 tokens, 16 heads x 72
+// 575 -> 42 us; 1024 tokens, 16 heads x 64 4047 -> 169 us (25 TFLOP/s); 64
+// tokens, 4 heads x 32 17.4 -> 5.1 us.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ long long tok_row(const AttnArgs& a, int b, int n) {
   return n < a.Nt ? (long long)b * a.Nt + n : (long long)a.B * a.Nt + (long long)b * a.Ni + (n - a.Nt);
 }
 
-template <class T>
-__global__ void __launch_bounds__(256) k_attn_simt(AttnArgs a, float scale) {
-  __shared__ float qs[8][128];
-  const int N = a.Nt + a.Ni;
-  const int h = blockIdx.y, b = blockIdx.z;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qi = blockIdx.x * 8 + warp;
-  if (qi >= N) return;
-  const T* Q = reinterpret_cast<const T*>(a.q);
-  const T* Kp = reinterpret_cast<const T*>(a.k);
-  const T* Vp = reinterpret_cast<const T*>(a.v);
-  const long long qr = tok_row(a, b, qi);
-  for (int e = lane; e < a.hd; e += 32) qs[warp][e] = to_f(Q[qr * a.ld_qkv + (size_t)h * a.hd + e]);
-  __syncwarp();
-  float m = -INFINITY, l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int c0 = 0; c0 < N; c0 += 32) {
-    const int key = c0 + lane;
-    float sc = -INFINITY;
-    if (key < N) {
-      const T* kr = Kp + tok_row(a, b, key) * a.ld_qkv + (size_t)h * a.hd;
-      float dot = 0.f;
-      for (int e = 0; e < a.hd; ++e) dot = fmaf(qs[warp][e], to_f(kr[e]), dot);
-      sc = dot * scale;
-    }
-    float cmax = sc;
+constexpr int FA_BQ = 32, FA_BK = 64, FA_THREADS = 128, FA_LDP = 80;  // P rows 80 apart: two groups' rows in distinct banks
+static size_t fa_smem(int hd) { return sizeof(float) * ((size_t)(FA_BQ + 2 * FA_BK) * (hd + 4) + FA_BQ * FA_LDP); }
+
+template <class T, int DG, bool VEC>
+__global__ void __launch_bounds__(FA_THREADS) k_attn_f32(AttnArgs a, float scale) {
+  extern __shared__ __align__(16) float sm[];
+  pdl_trigger();
+  const int N = a.Nt + a.Ni, hd = a.hd, ld = hd + 4;   // (hd + 4 = 4 x odd: eight rows' vectors in distinct banks)
+  float* const sQ = sm;
+  float* const sK = sQ + FA_BQ * ld;
+  float* const sV = sK + FA_BK * ld;
+  float* const sP = sV + FA_BK * ld;
+  const int h = blockIdx.y, b = blockIdx.z, q0 = blockIdx.x * FA_BQ;
+  const int tid = threadIdx.x, tk = tid & 15, tq = tid >> 4;
+  // rows n0 .. n0 + rows - 1 of the sample's head into s (zeros past N)
+  auto load = [&](const void* base, float* s, int n0, int rows) {
+    const T* g = reinterpret_cast<const T*>(base) + (size_t)h * hd;
+    constexpr int E = VEC ? VecN<T>::n : 1;
+    const int cpr = hd / E;
+    for (int c = tid; c < rows * cpr; c += FA_THREADS) {
+      const int r = c / cpr, e = (c % cpr) * E;
+      const bool in = n0 + r < N;
+      const T* src = in ? g + tok_row(a, b, n0 + r) * a.ld_qkv + e : g;
+      float* d = s + r * ld + e;
+      if constexpr (VEC && sizeof(T) == 4) {
+        cp16(d, src, in);
+      } else if constexpr (VEC) {
+        float v[VecN<T>::n];
+        ld16(src, v);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, off));
-    const float mn = fmaxf(m, cmax);
-    const float alpha = expf(m - mn);
-    const float p = key < N ? expf(sc - mn) : 0.f;
-    float psum = p;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, off);
-    l = l * alpha + psum;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) o[j] *= alpha;
-    const int nk = min(32, N - c0);
-    for (int j = 0; j < nk; ++j) {
-      const float pj = __shfl_sync(0xffffffffu, p, j);
-      const T* vr = Vp + tok_row(a, b, c0 + j) * a.ld_qkv + (size_t)h * a.hd;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int e = lane + 32 * q;
-        if (e < a.hd) o[q] = fmaf(pj, to_f(vr[e]), o[q]);
+        for (int z = 0; z < VecN<T>::n; ++z) d[z] = in ? v[z] : 0.f;
+      } else {
+        *d = in ? to_f(*src) : 0.f;
       }
     }
-    m = mn;
-  }
-  T* out = reinterpret_cast<T*>(a.out) + qr * a.ld_out + (size_t)h * a.hd;
-  const float inv = 1.0f / l;
+  };
+  const int nt = (N + FA_BK - 1) / FA_BK;
+  pdl_wait();
+  load(a.q, sQ, q0, FA_BQ);
+  load(a.k, sK, 0, FA_BK);
+  cp_commit();
+  load(a.v, sV, 0, FA_BK);
+  cp_commit();
+
+  float m[4], l[4], o[4][2 * DG];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int e = lane + 32 * q;
-    if (e < a.hd) out[e] = from_f<T>(o[q] * inv);
+  for (int i = 0; i < 4; ++i) {
+    m[i] = -INFINITY;
+    l[i] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 2 * DG; ++c) o[i][c] = 0.f;
+  }
+  const float* const qp = sQ + tq * ld;
+  const float* const kp = sK + tk * ld;
+  float* const pp = sP + tq * FA_LDP;
+  for (int t = 0; t < nt; ++t) {
+    cp_wait<1>();                                      // this tile's keys (its values may be in flight)
+    __syncthreads();
+    unsigned long long s2[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s2[i][j] = 0ull;
+#pragma unroll 2
+    for (int e = 0; e < hd; e += 4) {
+      ulonglong2 qv[4], kv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) qv[i] = *reinterpret_cast<const ulonglong2*>(qp + 8 * i * ld + e);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) kv[j] = *reinterpret_cast<const ulonglong2*>(kp + 16 * j * ld + e);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ffma2(s2[i][j], qv[i].x, kv[j].x);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ffma2(s2[i][j], qv[i].y, kv[j].y);
+    }
+    __syncthreads();                                   // the key buffer is free
+    if (t + 1 < nt) load(a.k, sK, (t + 1) * FA_BK, FA_BK);
+    cp_commit();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float s[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float dot = __uint_as_float((unsigned)s2[i][j]) + __uint_as_float((unsigned)(s2[i][j] >> 32));
+        s[j] = t * FA_BK + tk + 16 * j < N ? dot * scale : -INFINITY;
+      }
+      float cm = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, w));
+      const float mn = fmaxf(m[i], cm);
+      const float alpha = expf(m[i] - mn);
+      float ps = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float p = t * FA_BK + tk + 16 * j < N ? expf(s[j] - mn) : 0.f;
+        ps += p;
+        pp[8 * i * FA_LDP + tk + 16 * j] = p;
+      }
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, w);
+      l[i] = l[i] * alpha + ps;
+      m[i] = mn;
+#pragma unroll
+      for (int c = 0; c < 2 * DG; ++c) o[i][c] *= alpha;
+    }
+    cp_wait<1>();                                      // this tile's values
+    __syncthreads();
+#pragma unroll 2
+    for (int k = 0; k < FA_BK; k += 4) {
+      float4 p4[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) p4[i] = *reinterpret_cast<const float4*>(pp + 8 * i * FA_LDP + k);
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+#pragma unroll
+        for (int g = 0; g < DG; ++g) {
+          const int c = 2 * tk + 32 * g;
+          const float2 v = c < hd ? *reinterpret_cast<const float2*>(sV + (k + z) * ld + c) : make_float2(0.f, 0.f);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float p = z == 0 ? p4[i].x : z == 1 ? p4[i].y : z == 2 ? p4[i].z : p4[i].w;
+            o[i][2 * g] = fmaf(p, v.x, o[i][2 * g]);
+            o[i][2 * g + 1] = fmaf(p, v.y, o[i][2 * g + 1]);
+          }
+        }
+      }
+    }
+    __syncthreads();                                   // the value buffer is free
+    if (t + 1 < nt) load(a.v, sV, (t + 1) * FA_BK, FA_BK);
+    cp_commit();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int n = q0 + tq + 8 * i;
+    if (n >= N) continue;
+    const float inv = 1.0f / l[i];
+    T* out = reinterpret_cast<T*>(a.out) + tok_row(a, b, n) * a.ld_out + (size_t)h * hd;
+#pragma unroll
+    for (int g = 0; g < DG; ++g) {
+      const int c = 2 * tk + 32 * g;
+      if (c < hd) {
+        out[c] = from_f<T>(o[i][2 * g] * inv);
+        out[c + 1] = from_f<T>(o[i][2 * g + 1] * inv);
+      }
+    }
   }
 }
 
-cudaError_t attention_simt(DType dt, const AttnArgs& a, cudaStream_t s) {
-  const int N = a.Nt + a.Ni;
-  dim3 grid((N + 7) / 8, a.H, a.B);
-  const float scale = 1.0f / sqrtf((float)a.hd);
-  if (dt == F32) k_attn_simt<float><<<grid, 256, 0, s>>>(a, scale);
-  else k_attn_simt<bf16><<<grid, 256, 0, s>>>(a, scale);
+template <class T, int DG, bool VEC>
+static cudaError_t attn_f32_launch(const AttnArgs& a, cudaStream_t s) {
+  const size_t smem = fa_smem(a.hd);
+  const cudaError_t attr = cudaFuncSetAttribute(k_attn_f32<T, DG, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)fa_smem(32 * DG));
+  if (attr != cudaSuccess) return attr;
+  launch_pdl(k_attn_f32<T, DG, VEC>, dim3((a.Nt + a.Ni + FA_BQ - 1) / FA_BQ, a.H, a.B), dim3(FA_THREADS), smem, s, a,
+             1.0f / sqrtf((float)a.hd));
   return launched();
+}
+
+template <class T>
+static cudaError_t attn_f32_t(const AttnArgs& a, cudaStream_t s) {
+  // 16-byte copies need aligned head rows; hd is a multiple of 8
+  const bool vec = a.ld_qkv % VecN<T>::n == 0 && !(((uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v) & 15);
+#define FF_FA(dg) case dg: return vec ? attn_f32_launch<T, dg, true>(a, s) : attn_f32_launch<T, dg, false>(a, s);
+  switch ((a.hd + 31) / 32) {
+    FF_FA(1) FF_FA(2) FF_FA(3) FF_FA(4)
+    default: return cudaErrorInvalidValue;
+  }
+#undef FF_FA
+}
+
+cudaError_t attention_simt(DType dt, const AttnArgs& a, cudaStream_t s) {
+  return dt == F32 ? attn_f32_t<float>(a, s) : attn_f32_t<bf16>(a, s);
 }
 
 }  // namespace ff

@@ -47,3 +47,29 @@ def test_f32_gemm(cuda, M, N, K, fused):
     torch.cuda.synchronize()
     assert rel_l2(f64(out)[:M], ref) < TOL
     assert torch.all(out[M] == 7.0)
+
+
+# one and several tiles of 32 queries / 64 keys with remainders, text + image
+# rows, every width class of the output columns; row strides that are not
+# 16-byte multiples (scalar copies); bf16 head widths without a tensor-core
+# kernel.  An output is a convex combination of values off by a few u (fp32:
+# the exponents' error, |s| u, dominates) or by the storage rounding (bf16).
+F32_ATTN = [("f32", 1, 0, 64, 4, 32, 0), ("f32", 2, 7, 90, 2, 72, 8), ("f32", 1, 0, 1, 3, 8, 0),
+            ("f32", 2, 0, 256, 3, 72, 0), ("f32", 1, 33, 160, 2, 128, 4), ("f32", 3, 65, 1, 2, 64, 0),
+            ("f32", 1, 5, 130, 2, 40, 3), ("f32", 1, 0, 97, 1, 104, 1), ("bf16", 2, 5, 100, 2, 96, 0),
+            ("bf16", 1, 0, 70, 3, 40, 5), ("bf16", 1, 9, 200, 2, 8, 8)]
+
+
+@pytest.mark.parametrize("dtype,B,nt,ni,H,d,pad", F32_ATTN)
+def test_f32_attention(cuda, dtype, B, nt, ni, H, d, pad):
+    C, n = H * d, nt + ni
+    buf = randn((B * n, 3 * C + pad), dtype, 13)
+    out = torch.full((B * n + 1, C), 3.0, dtype=buf.dtype, device=cuda)
+    ff.featfix_op_attention(dtype, buf, out[:-1], B, nt, ni, H, d)
+    torch.cuda.synchronize()
+    rows = torch.tensor([[b * nt + t if t < nt else B * nt + b * ni + t - nt for t in range(n)] for b in range(B)])
+    x = torch.from_numpy(f64(buf))[rows]
+    q, k, v = (x[..., i * C:(i + 1) * C].reshape(B, n, H, d).transpose(1, 2) for i in range(3))
+    ref = (torch.softmax(q @ k.transpose(2, 3) / d ** 0.5, -1) @ v).transpose(1, 2).reshape(B, n, C)
+    assert rel_l2(f64(out)[rows], ref.numpy()) < (2e-6 if dtype == "f32" else 4e-3)
+    assert torch.all(out[-1] == 3.0)
