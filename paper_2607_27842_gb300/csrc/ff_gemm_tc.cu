@@ -108,9 +108,25 @@ struct TileAt {
   bool sw;
   int m0, n0;  // first output row / column
 };
+// Tile order: groups of GM row blocks, each swept over all column blocks with
+// its rows fastest, so the tiles running together cover about a square of the
+// output and a group's rows of A are read from DRAM once (with all row blocks
+// fastest, 14310 x 2048 x 8192 read its 234 MB of A for each of the 8 column
+// blocks: 1515 MB of DRAM traffic and 333 us, now 290 us).
+template <int GM>
+__device__ __forceinline__ void grouped_tile(int tile, int num_m, int num_n, int& m, int& n) {
+  const int g = tile / (GM * num_n), r = tile - g * GM * num_n;
+  const int gm = min(GM, num_m - g * GM);
+  n = r / gm;
+  m = g * GM + r - n * gm;
+}
 template <int BN>
 __device__ __forceinline__ TileAt tile_at(const TileMap& t, int tile) {
-  if (tile < t.n_norm) return {false, (tile % t.num_m) * BM, (tile / t.num_m) * BN};
+  if (tile < t.n_norm) {
+    int m, n;
+    grouped_tile<16>(tile, t.num_m, t.n_full, m, n);
+    return {false, m * BM, n * BN};
+  }
   const int u = tile - t.n_norm;
   return {true, (u % t.num_m2) * 256, t.n_full * BN + (u / t.num_m2) * 128};
 }
@@ -694,9 +710,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   auto tile_of = [&](int tile, bool& g1, int& mb, int& nb) {
     g1 = GROUPED && tile < n1;
     const int u = g1 ? tile : tile - n1;
-    const int nm = g1 ? num_m1 : num_m;
-    mb = u % nm;
-    nb = u / nm;
+    grouped_tile<8>(u, g1 ? num_m1 : num_m, num_n, mb, nb);
   };
   const int num_kb = (K + BK - 1) / BK;
 
@@ -928,19 +942,37 @@ bool staged_maps(const EpiArgs& e, int M, int N, CUtensorMap* mo, CUtensorMap* m
          (!e.hist_out || make_store_map(mh, e.hist_out, M, N, e.ldo));
 }
 
-// Tile width choice: the fewest waves of rows_per_tile x BN tiles over the
-// available CTAs (or CTA pairs), ties to the wider tile (less shared-memory
-// traffic per FLOP).
-int pick_bn(int M, int N, int rows_per_tile, int slots) {
-  double best = 1e30;
-  int bn = 256;
-  for (int cand : {256, 128}) {
-    const long long tiles = (long long)((M + rows_per_tile - 1) / rows_per_tile) * ((N + cand - 1) / cand);
-    const long long waves = (tiles + slots - 1) / slots;
-    const double cost = (double)waves * cand;
-    if (cost < best - 1e-9) { best = cost; bn = cand; }
-  }
-  return bn;
+// Tile width of the CTA-pair kernel, 0 where single CTAs are the better
+// choice.  m256, t128x256: 256-row blocks of A over the launch's problems, and
+// the single-CTA kernel's 128 x 256 tiles (its swapped remainder tiles
+// counted); act: the layer has an activation.  A pair's 256 x 256 tile and a
+// CTA's 128 x 256 tile take each SM about as long, the pair 5-20% less (each
+// CTA loads half of the W tile: 14310 x 6144 x 2048 219 -> 199 us, 4608 x 3072
+// x 2048 51 -> 43, 14310 x 2048 x 256 68 -> 58), so pairs run wherever they
+// need no more waves, with two exceptions: within one wave short reductions
+// stay with single CTAs, whose epilogue blocks come by TMA (1024 x 4608 x 256
+// 9.2 against 9.5 us), and so do short reductions with an activation, bound
+// by their epilogues (DiT-XL/2 sampling with its fc1 layers on pairs 54.4 ms,
+// on single CTAs 53.1).  128-wide pair tiles take 0.85 of a 256-wide tile's
+// time (both operands from shared memory: N = 128 runs at little more than
+// half rate), so they pay only where the 256-wide tiles leave half the pairs
+// idle; counted at half the time they took 8192 x 8192 x 8192, 945 us against
+// 590.
+int pair_bn(long long m256, long long t128x256, int N, int K, bool act, int sms) {
+  const int pairs = sms / 2;
+  const long long w_single = (t128x256 + sms - 1) / sms;
+  const long long w256 = (m256 * ((N + 255) / 256) + pairs - 1) / pairs;
+  const long long w128 = (m256 * ((N + 127) / 128) + pairs - 1) / pairs;
+  if (w256 > w_single) return 0;
+  if (w128 <= w256) return 128;
+  if (act && K < 1536) return 0;
+  return w256 > 1 || K >= 1024 ? 256 : 0;
+}
+
+// The single-CTA kernel's 128 x 256 tiles, remainder columns in swapped tiles.
+long long wide_tiles(int M, int N) {
+  const int rem = N % 256;
+  return (long long)((M + BM - 1) / BM) * (N / 256) + (rem ? (long long)((rem + 127) / 128) * ((M + 255) / 256) : 0);
 }
 
 }  // namespace
@@ -953,14 +985,9 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
   if (!ln_ok(e, N)) return cudaErrorInvalidValue;
   if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
-  // Long reductions: CTA pairs (256-row tiles, each CTA stages half of W);
-  // measured faster than single CTAs only from K of about 8k on.  (256 x 128
-  // pair tiles for the one-wave DiT-XL/2 layers, two tiles per pair so that
-  // an epilogue runs beside the next mainloop, measured slower: fc2 44.8 ->
-  // 49.8 us, out-projection 19.1 -> 18.0 us.)
-  if (M >= 2 * BM && K >= 8192) {
+  const int bn = M >= 2 * BM ? pair_bn((M + 2 * BM - 1) / (2 * BM), wide_tiles(M, N), N, K, e.act != 0, g_sms) : 0;
+  if (bn) {
     const int pairs = g_sms / 2;
-    const int bn = pick_bn(M, N, 2 * BM, pairs);
     if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, bn / 2)) return cudaErrorInvalidValue;
     const long long tiles = (long long)((M + 2 * BM - 1) / (2 * BM)) * ((N + bn - 1) / bn);
     const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
@@ -983,7 +1010,7 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
   tm.num_m = (M + BM - 1) / BM;
   tm.num_m2 = (M + 255) / 256;
   const int rem = N % 256;
-  const long long t256 = (long long)tm.num_m * (N / 256) + (rem ? (long long)((rem + 127) / 128) * tm.num_m2 : 0);
+  const long long t256 = wide_tiles(M, N);
   const long long t128 = (long long)tm.num_m * ((N + 127) / 128);
   const bool wide = (t256 + g_sms - 1) / g_sms <= (t128 + g_sms - 1) / g_sms;
   CUtensorMap mw128 = {}, ma256 = {}, mo = {}, mh = {}, mr = {}, mhb = {};
@@ -1059,15 +1086,15 @@ cudaError_t gemm_tc_grouped(int M0, const void* A0, const void* W0, const EpiArg
   if (!init_driver()) return cudaErrorNotSupported;
   if (!ln_ok(e0, N) || !ln_ok(e1, N) || (ln_side(e0) && ln_side(e1) && ln_side(e0) != ln_side(e1)))
     return cudaErrorInvalidValue;
-  // long reductions: both problems in one CTA-pair launch (256-row tiles
-  // of the image rows, then of the text rows)
-  if (M0 >= 2 * BM && K >= 8192) {
+  // both problems in one CTA-pair launch (256-row tiles of the text rows,
+  // then of the image rows)
+  const long long rows_t = ((M0 + 2 * BM - 1) / (2 * BM)) + ((M1 + 2 * BM - 1) / (2 * BM));
+  const int bn = M0 >= 2 * BM ? pair_bn(rows_t, wide_tiles(M0, N) + wide_tiles(M1, N), N, K, e0.act != 0, g_sms) : 0;
+  if (bn) {
     if (K % 8 != 0 || lda % 8 != 0 || ldw % 8 != 0 || N % 8 != 0) return cudaErrorInvalidValue;
     if (((uintptr_t)A0 & 15) || ((uintptr_t)W0 & 15) || ((uintptr_t)A1 & 15) || ((uintptr_t)W1 & 15))
       return cudaErrorInvalidValue;
     const int pairs = g_sms / 2;
-    const long long rows_t = ((M0 + 2 * BM - 1) / (2 * BM)) + ((M1 + 2 * BM - 1) / (2 * BM));
-    const int bn = pick_bn((int)(rows_t * 2 * BM), N, 2 * BM, pairs);
     CUtensorMap a0, b0, a1, b1;
     if (!make_map(&a0, A0, M0, K, lda, BM) || !make_map(&b0, W0, N, K, ldw, bn / 2) ||
         !make_map(&a1, A1, M1, K, lda, BM) || !make_map(&b1, W1, N, K, ldw, bn / 2))

@@ -1,0 +1,53 @@
+"""bf16 dense layers at the edges of the tile shapes and of the rules that pick
+them (single CTAs or CTA pairs, 128- or 256-wide tiles, several groups of row
+blocks), against float64."""
+
+import pytest
+import torch
+
+import oracle
+from paper_2607_27842_gb300 import featfix as ff
+
+from .gpu_helpers import rel_l2
+from .test_gpu_ops import f64, randn
+
+pytestmark = pytest.mark.gpu
+
+# M, N, K, rows per gate sample
+SHAPES = [(256, 32, 64, 256),        # pairs, one 128-wide tile, mostly empty
+          (257, 136, 72, 40),        # a second row block of one row, 8 remainder columns
+          (255, 256, 64, 255),       # one row short of a pair: single CTAs
+          (511, 264, 8, 32),         # one k-step of 8
+          (1024, 4608, 256, 256),    # one wave, short reduction: single CTAs
+          (1024, 4608, 1024, 200),   # one wave, pairs
+          (2300, 1800, 136, 500),    # nine row blocks: two groups, the last of one block
+          (4352, 3464, 72, 4352)]    # 17 row blocks, three waves
+
+
+# the result is stored in bf16 (2^-9 relative, 1.7e-3 in the norm), the
+# increment is the difference of two stored values rounded again
+@pytest.mark.parametrize("M,N,K,rpb", SHAPES)
+@pytest.mark.parametrize("epilogue", ["bias", "gelu", "gated", "gated_history"])
+def test_gemm_tiles(cuda, M, N, K, rpb, epilogue):
+    a, w, bias = randn((M, K), "bf16", 1), randn((N, K), "bf16", 2, 0.1), randn(N, "bf16", 3)
+    buf = torch.full((M + 1, N), 5.0, dtype=torch.bfloat16, device=cuda)
+    out, kw, hist = buf[:M], {}, None
+    y = f64(a) @ f64(w).T + f64(bias)
+    if epilogue == "gelu":
+        kw = dict(act=1)
+        y = oracle.model.gelu_tanh(y)
+    if epilogue.startswith("gated"):
+        gate = randn((-(-M // rpb), 2 * N), "f32", 7)
+        resid = randn((M, N), "bf16", 8)
+        kw = dict(gate=gate[:, N:], gate_stride=2 * N, rows_per_batch=rpb, resid=resid)
+        y = f64(resid) + f64(gate)[torch.arange(M).numpy() // rpb, N:] * y
+    if epilogue == "gated_history":
+        base, hist = randn((M, N), "bf16", 9), torch.full((M + 1, N), 5.0, dtype=torch.bfloat16, device=cuda)
+        kw.update(hist_base=base, hist_out=hist[:M])
+    ff.featfix_op_gemm("bf16", a, w, out, bias=bias, **kw)
+    torch.cuda.synchronize()
+    assert rel_l2(f64(out), y) < 4e-3
+    assert torch.all(buf[M] == 5.0)
+    if hist is not None:
+        assert rel_l2(f64(hist)[:M], f64(out) - f64(base)) < 4e-3
+        assert torch.all(hist[M] == 5.0)
