@@ -166,23 +166,6 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// packed pairs of fp32 (one 64-bit register pair): a.x + 2^32 * a.y
-__device__ __forceinline__ unsigned long long f2u(float a, float b) {
-  return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
-}
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fadd2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ float lo_f(unsigned long long x) { return __uint_as_float((unsigned)x); }
-__device__ __forceinline__ float hi_f(unsigned long long x) { return __uint_as_float((unsigned)(x >> 32)); }
-
 // 16 pairs of S (v[2e], v[2e + 1]) -> exp2(s * scale - m) as bf16 pairs,
 // their sum added to the packed accumulators
 __device__ __forceinline__ void exp_pairs16(const float* v, unsigned long long sc2, unsigned long long nm2,

@@ -71,11 +71,16 @@ __device__ __forceinline__ float gelu_tanh(float x) {
 }
 // Same GELU through the hardware tanh approximation (tanh.approx.f32, about
 // 2^-11 relative error): for bf16 outputs, whose rounding is 2^-9.
-__device__ __forceinline__ float gelu_tanh_fast(float x) {
-  const float k0 = 0.7978845608028654f;
+// (fma form, the same operations as the packed pairs of the staged epilogue)
+__device__ __forceinline__ float tanh_approx(float x) {
   float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(k0 * (x + 0.044715f * x * x * x)));
-  return 0.5f * x * (1.0f + t);
+  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(x));
+  return t;
+}
+constexpr float GELU_K0 = 0.7978845608028654f, GELU_K1 = 0.7978845608028654f * 0.044715f;
+__device__ __forceinline__ float gelu_tanh_fast(float x) {
+  const float h = 0.5f * x;
+  return __fmaf_rn(h, tanh_approx(x * __fmaf_rn(x * x, GELU_K1, GELU_K0)), h);
 }
 __device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
 
@@ -153,13 +158,18 @@ __device__ __forceinline__ void epi_rope_act(const EpiArgs& e, int m, int n0, fl
   if (e.rope && m >= e.rope_row0 && n0 < e.rope_cols) {
     const int tok = (m - e.rope_row0) % e.rope_period;
     const int half = e.rope_hd >> 1;
+    // two pairs per 16-byte load: head widths are multiples of 8, so pairs j and
+    // j + 1 of an even j lie in one head and on 16 bytes
+    static_assert(CH % 4 == 0, "whole 16-byte loads");
 #pragma unroll
-    for (int j = 0; j < CH; j += 2) {
+    for (int j = 0; j < CH; j += 4) {
       const int pair = ((n0 + j) % e.rope_hd) >> 1;
-      const float2 cs = e.rope[(size_t)tok * half + pair];
-      const float a = v[j], b = v[j + 1];
+      const float4 cs = *reinterpret_cast<const float4*>(e.rope + (size_t)tok * half + pair);
+      const float a = v[j], b = v[j + 1], c = v[j + 2], d = v[j + 3];
       v[j] = a * cs.x - b * cs.y;
       v[j + 1] = a * cs.y + b * cs.x;
+      v[j + 2] = c * cs.z - d * cs.w;
+      v[j + 3] = c * cs.w + d * cs.z;
     }
   }
   if (e.act == 1 && n0 >= e.act_col0) {

@@ -104,6 +104,15 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 __device__ __forceinline__ float2 unpack2(uint32_t u) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
 }
+// gelu_tanh_fast on 16 packed pairs
+__device__ __forceinline__ void gelu_pairs(unsigned long long (&y)[16]) {
+  const unsigned long long k0 = f2u(GELU_K0, GELU_K0), k1 = f2u(GELU_K1, GELU_K1), hf = f2u(0.5f, 0.5f);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const unsigned long long in = fmul2(y[i], ffma2(fmul2(y[i], y[i]), k1, k0)), hx = fmul2(y[i], hf);
+    y[i] = ffma2(hx, f2u(tanh_approx(lo_f(in)), tanh_approx(hi_f(in))), hx);
+  }
+}
 struct TileAt {
   bool sw;
   int m0, n0;  // first output row / column
@@ -142,6 +151,14 @@ struct EpiWarp {
   int warp, lane, q, h, row, c_lo;
 };
 
+// The epilogue comes in three forms, a kernel instance each, so that none pays
+// registers or branches for the others:
+//   EPI_FULL    gate, residual, history increment (any of them);
+//   EPI_PLAIN   bias, RoPE, activation only (qkv, fc1, linear1);
+//   EPI_SINGLE  EPI_FULL with a residual where every CTA holds one tile, so
+//               nothing hides the epilogue (epi_single below).
+enum { EPI_FULL = 0, EPI_PLAIN = 1, EPI_SINGLE = 2 };
+
 // The epilogue of one tile, inlined once per problem of the launch so that
 // every EpiArgs / TileMap field and tensor map is read from its own kernel
 // parameter (a run-time choice between two parameter structs turns every
@@ -149,7 +166,7 @@ struct EpiWarp {
 // tiles without residual preloads (the second problem of a grouped launch,
 // the CTA pairs).  XB: bytes of the epilogue warps' staging buffers (0: the
 // per-lane store path only).  Returns false when the accumulator wait gave up.
-template <int BN, int XB, bool PLAIN, int LN>
+template <int BN, int XB, bool PLAIN, int LN, int EPI>
 __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, const TileMap& tm, const int M,
                                          const int N, const TileAt t, const int acc, const uint32_t aph,
                                          uint32_t& epi_cnt, const CUtensorMap* tmO, const CUtensorMap* tmH,
@@ -162,7 +179,7 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
   uint64_t* const tfull = W.tfull;
   volatile int* const abort_flag = W.abort_flag;
   const uint32_t tmem_base = W.tmem_base;
-  const int pre = PLAIN ? 0 : tm.pre;
+  const int pre = PLAIN || LN == 0 ? 0 : tm.pre;
   constexpr int LNM = LN == 1 ? 1 : LN == 2 ? 2 : 0;
   const bool sw = !PLAIN && t.sw;
   uint4 pr[4], ph[4];
@@ -193,7 +210,30 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
                    : make_uint4(0, 0, 0, 0);
     }
   };
-  if (XB > 0 && tm.staged && !sw) fetch(t.n0 + c_lo);
+  // EPI_PLAIN: the chunk's bias in 16-byte loads, the same for every lane (one
+  // sector each), a chunk ahead
+  uint4 bv4[4];
+  const bool bias_al = !((uintptr_t)e.bias & 15);
+  auto fetch_bias = [&](int n0) {
+    const bf16* bp = reinterpret_cast<const bf16*>(e.bias) + n0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (!e.bias || n0 + 8 * k >= N) {
+        bv4[k] = make_uint4(0, 0, 0, 0);
+      } else if (bias_al) {
+        bv4[k] = *reinterpret_cast<const uint4*>(bp + 8 * k);
+      } else {
+        const unsigned short* us = reinterpret_cast<const unsigned short*>(bp + 8 * k);
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = (uint32_t)us[2 * i] | ((uint32_t)us[2 * i + 1] << 16);
+        bv4[k] = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+  };
+  if (XB > 0 && tm.staged && !sw) {
+    if constexpr (EPI == EPI_PLAIN) fetch_bias(t.n0 + c_lo); else fetch(t.n0 + c_lo);
+  }
   int ok = 1;
   if (lane == 0) ok = mbar_wait_g(&tfull[acc], aph, abort_flag) ? 1 : 0;
   ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -236,6 +276,54 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
         const float2 st = epi_chunk<bf16, 32, LNM>(e, m, n0, N, v, lnr);
         if ((LN == 2 && e.ln_out)) ln_put(e, m, n0, st);
       }
+    }
+  } else if (EPI == EPI_PLAIN && !sw) {
+    // Staged epilogue of a layer without gate, residual and history: as
+    // below, in packed fp32 pairs and without shuffles (the costliest
+    // instructions beside a mainloop): 4096 x 4608 x 1152 with GELU 39.7 -> 33.6
+    // us, 14310 x 8192 x 2048 302 -> 273
+    const int m = t.m0 + row;
+    for (int c = c_lo; c < c_lo + BN / 2; c += 32) {
+      const int n0 = t.n0 + c;
+      if (n0 >= N) break;
+      float v[32];
+      tmem_ld32(tq + (uint32_t)c, v);
+      unsigned long long y[16];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t bb[4] = {bv4[k].x, bv4[k].y, bv4[k].z, bv4[k].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          y[4 * k + i] = fadd2(f2u(v[8 * k + 2 * i], v[8 * k + 2 * i + 1]), bf2u(bb[i]));
+      }
+      if (c + 32 < c_lo + BN / 2 && n0 + 32 < N) fetch_bias(n0 + 32);
+      if (e.act == 1 && !e.rope && n0 >= e.act_col0) {
+        gelu_pairs(y);
+      } else if (e.rope || e.act) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          v[2 * i] = lo_f(y[i]);
+          v[2 * i + 1] = hi_f(y[i]);
+        }
+        if (m < M) epi_rope_act<bf16, 32>(e, m, n0, v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) y[i] = f2u(v[2 * i], v[2 * i + 1]);
+      }
+      uint8_t* b0 = ep + (epi_cnt & 1) * 2048;
+      if (lane == 0) bulk_wait_read<1>();
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<uint4*>(b0 + blk_off(lane, k)) =
+            make_uint4(pack2(lo_f(y[4 * k]), hi_f(y[4 * k])), pack2(lo_f(y[4 * k + 1]), hi_f(y[4 * k + 1])),
+                       pack2(lo_f(y[4 * k + 2]), hi_f(y[4 * k + 2])), pack2(lo_f(y[4 * k + 3]), hi_f(y[4 * k + 3])));
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        tma_store(tmO, b0, n0, t.m0 + q * 32);
+        bulk_commit();
+      }
+      ++epi_cnt;
     }
   } else if (!sw) {
     // Staged epilogue: each 32-row x 32-column chunk is written into a
@@ -472,12 +560,195 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
   return true;
 }
 
+// First row past the sample of row r.
+__device__ __forceinline__ int sample_end(const EpiArgs& e, int r) {
+  if (r < e.seg_split) return min((r / e.rpb0 + 1) * e.rpb0, e.seg_split);
+  return e.seg_split + ((r - e.seg_split) / e.rpb1 + 1) * e.rpb1;
+}
+
+// Epilogue of the one tile of a CTA: out = resid + gate * act(acc + bias), and
+// the history increment.  Nothing runs beside it, so it is all latency: the
+// warp's residual blocks (32 x 32 bf16, 64-byte swizzle) are replaced by the
+// output in place and stored from there, one buffer per block, so no block
+// waits for another's store; two of them, the bias and the gate arrive
+// during the mainloop, the other blocks in the idle ring after it.  Normal tile:
+// lane = row, bias and gate broadcast from shared memory.  Swapped tile: lane =
+// column, so bias and gate stay in registers and each row of a block is one
+// 64-byte read and write, with no transposition buffer.
+// Against the shared form with its block-by-block buffers, shuffled bias and
+// gate and transposed swapped tiles: 4096 x 1152 x 1152 (gate, residual) 19.3
+// -> 14.5 us, 4096 x 1152 x 4608 (and history) 46.2 -> 42.6 us.
+template <int BN>
+__device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, const int M, const int N, const TileAt t,
+                                           const CUtensorMap* tmO, const CUtensorMap* tmH, const CUtensorMap* tmR,
+                                           const CUtensorMap* tmHB) {
+  const int lane = W.lane, q = W.q, h = W.h;
+  uint8_t* const ep = W.ep;
+  uint8_t* const ring = W.smem + (W.warp - 2) * 16384;    // 12 KB of blocks, 1.5 KB of constants
+  uint64_t* const rbar = &W.rbar[W.warp - 2];
+  const bool hist = e.hist_out != nullptr;
+  // block i: output rows y0 .. y0 + 31, columns x0 .. x0 + 31
+  const int xb = t.sw ? t.n0 + q * 32 : t.n0 + W.c_lo, yb = t.sw ? t.m0 + h * (BN / 2) : t.m0 + q * 32;
+  const int dx = t.sw ? 0 : 32, dy = t.sw ? 32 : 0;
+  const int nb = xb < N && yb < M ? min(4, t.sw ? (M - yb + 31) >> 5 : (N - xb + 31) >> 5) : 0;
+  auto rblk = [&](int i) { return i < 2 ? ep + i * 2048 : ring + (i - 2) * 2048; };
+  auto hblk = [&](int i) { return ring + 4096 + i * 2048; };
+  const int early = min(nb, 2);
+  if (lane == 0 && nb > 0) {
+    mbar_expect_tx(rbar, early * 2048u);
+    for (int i = 0; i < early; ++i) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
+  }
+  // bias and gate: normal tile, columns xb + 32 i + lane, samples of the warp's
+  // first and last row; swapped tile, column xb + lane, samples of block i's
+  // first and last row (at most two samples in 32 rows)
+  float cb[4], c0[4], c1[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int col = xb + i * dx + lane;
+    const int r0 = min(yb + i * dy, M - 1), r1 = min(yb + i * dy + 31, M - 1);
+    const bool in = i < nb && col < N;
+    cb[i] = in && e.bias ? __bfloat162float(reinterpret_cast<const bf16*>(e.bias)[col]) : 0.f;
+    c0[i] = in && e.gate ? e.gate[(size_t)epi_batch(e, r0) * e.gate_stride + col] : 1.f;
+    c1[i] = in && e.gate ? e.gate[(size_t)epi_batch(e, r1) * e.gate_stride + col] : 1.f;
+  }
+  int ok = 1;
+  if (lane == 0) {
+    ok = mbar_wait_g(W.tfull, 0, W.abort_flag) ? 1 : 0;
+    if (nb > 0) {  // the early blocks (they land before the CTA exits, also after a failed wait)
+      const unsigned long long t0 = gtimer();
+      while (!mbar_try(rbar, 0))
+        if (gtimer() - t0 > WAIT_LIMIT_NS) { atomicOr(&g_watchdog, 2u); *W.abort_flag = 1; ok = 0; break; }
+    }
+  }
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  if (!ok) return false;
+  tc_fence_after();
+  const bool late = nb > 2 || (hist && nb > 0);
+  if (lane == 0 && late) {
+    mbar_expect_tx(rbar, (uint32_t)((nb - early) + (hist ? nb : 0)) * 2048u);
+    for (int i = 0; i < nb; ++i) {
+      if (hist) tma_load(tmHB, rbar, hblk(i), xb + i * dx, yb + i * dy);
+      if (i >= 2) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
+    }
+  }
+  bool late_wait = late;
+  auto late_ready = [&]() -> bool {
+    if (!late_wait) return true;
+    late_wait = false;
+    int w = 1;
+    if (lane == 0) w = mbar_wait_g(rbar, 1, W.abort_flag) ? 1 : 0;
+    return __shfl_sync(0xffffffffu, w, 0) != 0;
+  };
+  const uint32_t tq = W.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * (BN / 2));
+  auto store = [&](int i) {
+    fence_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+      tma_store(tmO, rblk(i), xb + i * dx, yb + i * dy);
+      if (hist) tma_store(tmH, hblk(i), xb + i * dx, yb + i * dy);
+      bulk_commit();
+    }
+  };
+  if (!t.sw) {
+    float* const cst = reinterpret_cast<float*>(ring + 12288);   // bias [128], gate of the first and last row's sample
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      cst[32 * i + lane] = cb[i];
+      cst[128 + 32 * i + lane] = c0[i];
+      cst[256 + 32 * i + lane] = c1[i];
+    }
+    __syncwarp();
+    const int r0 = min(yb, M - 1), m = min(yb + lane, M - 1);
+    const float* const gp = cst + (e.gate && epi_batch(e, m) != epi_batch(e, r0) ? 256 : 128);
+    for (int i = 0; i < nb; ++i) {
+      float v[32];
+      tmem_ld32(tq + (uint32_t)(32 * i), v);
+      unsigned long long y[16];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const ulonglong2 b2 = *reinterpret_cast<const ulonglong2*>(cst + 32 * i + 4 * k);
+        y[2 * k] = fadd2(f2u(v[4 * k], v[4 * k + 1]), b2.x);
+        y[2 * k + 1] = fadd2(f2u(v[4 * k + 2], v[4 * k + 3]), b2.y);
+      }
+      if (e.act == 1) gelu_pairs(y);
+      if (e.gate) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const ulonglong2 g2 = *reinterpret_cast<const ulonglong2*>(gp + 32 * i + 4 * k);
+          y[2 * k] = fmul2(y[2 * k], g2.x);
+          y[2 * k + 1] = fmul2(y[2 * k + 1], g2.y);
+        }
+      }
+      if ((hist || i >= 2) && !late_ready()) return false;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        uint4* const rp = reinterpret_cast<uint4*>(rblk(i) + blk_off(lane, k));
+        const uint4 r4 = *rp;
+        const uint32_t rr[4] = {r4.x, r4.y, r4.z, r4.w};
+        uint32_t ob[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const unsigned long long a = fadd2(y[4 * k + z], bf2u(rr[z]));
+          ob[z] = pack2(lo_f(a), hi_f(a));
+        }
+        *rp = make_uint4(ob[0], ob[1], ob[2], ob[3]);
+        if (hist) {  // stored(out) - hist_base
+          uint4* const hp = reinterpret_cast<uint4*>(hblk(i) + blk_off(lane, k));
+          const uint4 h4 = *hp;
+          const uint32_t hh[4] = {h4.x, h4.y, h4.z, h4.w};
+          uint32_t hb[4];
+#pragma unroll
+          for (int z = 0; z < 4; ++z) {
+            const float2 o2 = unpack2(ob[z]), h2 = unpack2(hh[z]);
+            hb[z] = pack2(o2.x - h2.x, o2.y - h2.y);
+          }
+          *hp = make_uint4(hb[0], hb[1], hb[2], hb[3]);
+        }
+      }
+      store(i);
+    }
+  } else {
+    uint32_t off[4];   // byte of column `lane` in a block row r with (r >> 1) & 3 = x
+#pragma unroll
+    for (int x = 0; x < 4; ++x) off[x] = (uint32_t)((((lane >> 3) ^ x) << 4) + (lane & 7) * 2);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i >= nb) break;
+      float v[32];
+      tmem_ld32(tq + (uint32_t)(32 * i), v);   // v[j] = acc[yb + 32 i + j][xb + lane]
+      const int y0 = yb + 32 * i;
+      const int jb = sample_end(e, y0) - y0;   // rows from jb on: the second sample's gate
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] += cb[i];
+      if (e.act == 1) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = gelu_tanh_fast(v[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] *= j < jb ? c0[i] : c1[i];
+      if ((hist || i >= 2) && !late_ready()) return false;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        bf16* const rp = reinterpret_cast<bf16*>(rblk(i) + j * 64 + off[(j >> 1) & 3]);
+        const bf16 o = __float2bfloat16_rn(v[j] + __bfloat162float(*rp));
+        *rp = o;
+        if (hist) {
+          bf16* const hp = reinterpret_cast<bf16*>(hblk(i) + j * 64 + off[(j >> 1) & 3]);
+          *hp = __float2bfloat16_rn(__bfloat162float(o) - __bfloat162float(*hp));
+        }
+      }
+      store(i);
+    }
+  }
+  return true;
+}
+
 // GROUPED: a second problem (group 1, tm1.n_tiles > 0) of the same N and K
 // with its own A, W, rows and epilogue (the text stream of a two-stream
 // block beside the image stream), its tiles first in the tile list; both
 // groups then have only normal tiles and no residual preloads.  Without
 // GROUPED the group-1 parameters are unused.
-template <int BN, bool GROUPED, int LN>
+template <int BN, bool GROUPED, int LN, int EPI>
 __global__ void __launch_bounds__(THREADS, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               const __grid_constant__ CUtensorMap tmW128, const __grid_constant__ CUtensorMap tmA256,
@@ -624,13 +895,15 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1;
       bool ok;
-      if constexpr (GROUPED) {
-        ok = tile < n1 ? epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN>(W, e1, tm1, M1, N, tile_at<BN>(tm1, tile), acc, aph, epi_cnt, &tmO1,
+      if constexpr (EPI == EPI_SINGLE) {
+        ok = epi_single<BN>(W, e0, M0, N, tile_at<BN>(tm0, tile), &tmO, &tmH, &tmR, &tmHB);
+      } else if constexpr (GROUPED) {
+        ok = tile < n1 ? epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN, EPI>(W, e1, tm1, M1, N, tile_at<BN>(tm1, tile), acc, aph, epi_cnt, &tmO1,
                                             &tmH1, &tmR, &tmHB)
-                       : epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile - n1), acc, aph, epi_cnt, &tmO,
+                       : epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN, EPI>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile - n1), acc, aph, epi_cnt, &tmO,
                                             &tmH, &tmR, &tmHB);
       } else {
-        ok = epi_tile<BN, Cfg<BN>::XPOSE_BYTES, false, LN>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile), acc, aph, epi_cnt, &tmO, &tmH, &tmR,
+        ok = epi_tile<BN, Cfg<BN>::XPOSE_BYTES, false, LN, EPI>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile), acc, aph, epi_cnt, &tmO, &tmH, &tmR,
                                  &tmHB);
       }
       if (!ok) break;
@@ -677,7 +950,7 @@ template <int BN> struct Cfg2 {
 // epilogue and store maps: the text stream of a two-stream block beside the
 // image stream), its tiles first in the tile list, so its few tiles fill the
 // first problem's last wave instead of running alone on a handful of SMs.
-template <int BN, int LN, bool GROUPED>
+template <int BN, int LN, bool GROUPED, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     k_gemm_tc2(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmH, int M, int N, int K,
@@ -826,10 +1099,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       const TileAt t = {false, mb * 2 * BM + (int)rank * BM, nb * BN};
       bool ok;
       if (g1)
-        ok = epi_tile<BN, C::XPOSE_BYTES, true, LN>(W, e1, tm1, M1, N, t, acc, aph, epi_cnt, &tmO1, &tmH1, &tmO1,
+        ok = epi_tile<BN, C::XPOSE_BYTES, true, LN, EPI>(W, e1, tm1, M1, N, t, acc, aph, epi_cnt, &tmO1, &tmH1, &tmO1,
                                                      &tmO1);
       else
-        ok = epi_tile<BN, C::XPOSE_BYTES, true, LN>(W, e, tm, M, N, t, acc, aph, epi_cnt, &tmO, &tmH, &tmO, &tmO);
+        ok = epi_tile<BN, C::XPOSE_BYTES, true, LN, EPI>(W, e, tm, M, N, t, acc, aph, epi_cnt, &tmO, &tmH, &tmO, &tmO);
       if (!ok) break;
       tc_fence_before();
       mbar_arrive_cluster(map_to(&tempty[acc], 0));
@@ -849,15 +1122,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-// k_gemm_tc instance for a fused-LayerNorm side (0 none, 1 consumer, 2 producer)
+// Kernel instance for a fused-LayerNorm side (0 none, 1 consumer, 2 producer)
+// and an epilogue form (the fused sides have the full one only).
 template <int BN, bool G>
-auto gemm_fn(int ln) -> decltype(&k_gemm_tc<BN, G, 0>) {
-  return ln == 1 ? k_gemm_tc<BN, G, 1> : ln == 2 ? k_gemm_tc<BN, G, 2> : k_gemm_tc<BN, G, 0>;
+auto gemm_fn(int ln, int epi) -> decltype(&k_gemm_tc<BN, G, 0, EPI_FULL>) {
+  if (ln == 1) return k_gemm_tc<BN, G, 1, EPI_FULL>;
+  if (ln == 2) return k_gemm_tc<BN, G, 2, EPI_FULL>;
+  if constexpr (BN == 256) {
+    if (epi == EPI_PLAIN) return k_gemm_tc<BN, G, 0, EPI_PLAIN>;
+    if constexpr (!G)
+      if (epi == EPI_SINGLE) return k_gemm_tc<BN, G, 0, EPI_SINGLE>;
+  }
+  return k_gemm_tc<BN, G, 0, EPI_FULL>;
 }
 template <int BN, bool G = false>
-auto gemm2_fn(int ln) -> decltype(&k_gemm_tc2<BN, 0, G>) {
-  return ln == 1 ? k_gemm_tc2<BN, 1, G> : ln == 2 ? k_gemm_tc2<BN, 2, G> : k_gemm_tc2<BN, 0, G>;
+auto gemm2_fn(int ln, int epi) -> decltype(&k_gemm_tc2<BN, 0, G, EPI_FULL>) {
+  if (ln == 1) return k_gemm_tc2<BN, 1, G, EPI_FULL>;
+  if (ln == 2) return k_gemm_tc2<BN, 2, G, EPI_FULL>;
+  return epi == EPI_PLAIN ? k_gemm_tc2<BN, 0, G, EPI_PLAIN> : k_gemm_tc2<BN, 0, G, EPI_FULL>;
 }
+int epi_form(const EpiArgs& e) { return e.gate || e.resid || e.hist_out ? EPI_FULL : EPI_PLAIN; }
 int ln_side(const EpiArgs& e) { return e.ln_in ? 1 : e.ln_out ? 2 : 0; }
 // a fused LayerNorm side: one side per launch, bf16 output of whole
 // 32-column chunks for the producer, 16-byte aligned rows everywhere
@@ -889,17 +1173,19 @@ bool init_driver() {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
     if (g_sms <= 0) g_sms = 148;
-    for (int ln = 0; ln < 3; ++ln) {
-      cudaFuncSetAttribute(gemm_fn<128, false>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<128>::SMEM);
-      cudaFuncSetAttribute(gemm_fn<256, false>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<256>::SMEM);
-      cudaFuncSetAttribute(gemm_fn<256, true>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<256>::SMEM);
-    }
-    for (int ln = 0; ln < 3; ++ln) {
-      cudaFuncSetAttribute(gemm2_fn<128>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg2<128>::SMEM);
-      cudaFuncSetAttribute(gemm2_fn<256>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg2<256>::SMEM);
-      cudaFuncSetAttribute(gemm2_fn<128, true>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg2<128>::SMEM);
-      cudaFuncSetAttribute(gemm2_fn<256, true>(ln), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg2<256>::SMEM);
-    }
+    auto smem = [](const void* fn, size_t bytes) {
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    for (int ln = 0; ln < 3; ++ln)
+      for (int epi : {EPI_FULL, EPI_PLAIN, EPI_SINGLE}) {
+        smem((const void*)gemm_fn<128, false>(ln, epi), Cfg<128>::SMEM);
+        smem((const void*)gemm_fn<256, false>(ln, epi), Cfg<256>::SMEM);
+        smem((const void*)gemm_fn<256, true>(ln, epi), Cfg<256>::SMEM);
+        smem((const void*)gemm2_fn<128>(ln, epi), Cfg2<128>::SMEM);
+        smem((const void*)gemm2_fn<256>(ln, epi), Cfg2<256>::SMEM);
+        smem((const void*)gemm2_fn<128, true>(ln, epi), Cfg2<128>::SMEM);
+        smem((const void*)gemm2_fn<256, true>(ln, epi), Cfg2<256>::SMEM);
+      }
   });
   return g_encode != nullptr;
 }
@@ -996,10 +1282,10 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
     tm2.staged = staged_maps(e, M, N, &mo, &mh) ? 1 : 0;
     const TileMap none = {};
     if (bn == 256)
-      launch_pdl(gemm2_fn<256>(ln_side(e)), grid, THREADS, Cfg2<256>::SMEM, s, ma, mb, mo, mh, M, N, K, tm2, e, ma, mb,
+      launch_pdl(gemm2_fn<256>(ln_side(e), epi_form(e)), grid, THREADS, Cfg2<256>::SMEM, s, ma, mb, mo, mh, M, N, K, tm2, e, ma, mb,
                  mo, mh, 0, none, e);
     else
-      launch_pdl(gemm2_fn<128>(ln_side(e)), grid, THREADS, Cfg2<128>::SMEM, s, ma, mb, mo, mh, M, N, K, tm2, e, ma, mb,
+      launch_pdl(gemm2_fn<128>(ln_side(e), epi_form(e)), grid, THREADS, Cfg2<128>::SMEM, s, ma, mb, mo, mh, M, N, K, tm2, e, ma, mb,
                  mo, mh, 0, none, e);
     return launched();
   }
@@ -1023,24 +1309,18 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
     if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, 256)) return cudaErrorInvalidValue;
     if (rem && (!make_map(&mw128, W, N, K, ldw, BM) || !make_map(&ma256, A, M, K, lda, 256)))
       return cudaErrorInvalidValue;
-    // staged (TMA-store) epilogue: one bf16 output of 16-byte aligned rows,
-    // plus the history stream when present
-    const bool aligned = !((uintptr_t)e.out & 15) && e.ldo % 8 == 0 &&
-                         (!e.hist_out || (!((uintptr_t)e.hist_out & 15) && !((uintptr_t)e.hist_base & 15)));
-    // (a warp's 32 rows must span at most two gate rows)
-    const bool gate_ok = !e.gate || ((e.seg_split <= 0 || e.rpb0 >= 32) && e.rpb1 >= 32);
-    if (!e.out_f32 && e.split_col >= N && aligned && gate_ok && make_store_map(&mo, e.out, M, N, e.ldo) &&
-        (!e.hist_out || make_store_map(&mh, e.hist_out, M, N, e.ldo)))
-      tm.staged = 1;
-    // one tile per CTA: residual / history-base blocks by TMA into the idle
-    // ring (16-byte aligned rows; otherwise the per-lane loads stay)
+    tm.staged = staged_maps(e, M, N, &mo, &mh) ? 1 : 0;
+    // one tile per CTA: residual / history-base blocks by TMA (16-byte aligned
+    // rows; otherwise the per-lane loads stay)
+    int epi = epi_form(e);
     if (tm.staged && t256 <= g_sms) {
       if (e.resid && make_store_map(&mr, const_cast<void*>(e.resid), M, N, e.ld_resid)) tm.pre |= 1;
       if (e.hist_out && make_store_map(&mhb, const_cast<void*>(e.hist_base), M, N, e.ldo)) tm.pre |= 2;
+      if ((tm.pre & 1) && (!e.hist_out || (tm.pre & 2)) && !e.rope && e.act != 2 && e.act_col0 == 0) epi = EPI_SINGLE;
     }
     const int grid = (int)(t256 < g_sms ? t256 : g_sms);
     const TileMap none = {};
-    launch_pdl(gemm_fn<256, false>(ln_side(e)), grid, THREADS, Cfg<256>::SMEM, s, ma, mb, mw128, ma256, mo, mh, mr, mhb, M, N, K, tm,
+    launch_pdl(gemm_fn<256, false>(ln_side(e), epi), grid, THREADS, Cfg<256>::SMEM, s, ma, mb, mw128, ma256, mo, mh, mr, mhb, M, N, K, tm,
                e, ma, mb, mo, mh, 0, none, e);
   } else {
     tm.n_full = (N + 127) / 128;
@@ -1049,7 +1329,7 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
     if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, 128)) return cudaErrorInvalidValue;
     const int grid = (int)(t128 < g_sms ? t128 : g_sms);
     const TileMap none = {};
-    launch_pdl(gemm_fn<128, false>(ln_side(e)), grid, THREADS, Cfg<128>::SMEM, s, ma, mb, ma, mb, ma, mb, ma, mb, M, N, K, tm, e, ma,
+    launch_pdl(gemm_fn<128, false>(ln_side(e), EPI_FULL), grid, THREADS, Cfg<128>::SMEM, s, ma, mb, ma, mb, ma, mb, ma, mb, M, N, K, tm, e, ma,
                mb, ma, mb, 0, none, e);
   }
   return launched();
@@ -1069,12 +1349,7 @@ bool group_maps(int M, int N, int K, const void* A, int lda, const void* W, int 
   if (!make_map(ma, A, M, K, lda, BM) || !make_map(mb, W, N, K, ldw, 256)) return false;
   *mo = *ma;
   *mh = *ma;
-  const bool aligned = !((uintptr_t)e.out & 15) && e.ldo % 8 == 0 &&
-                       (!e.hist_out || (!((uintptr_t)e.hist_out & 15) && !((uintptr_t)e.hist_base & 15)));
-  const bool gate_ok = !e.gate || ((e.seg_split <= 0 || e.rpb0 >= 32) && e.rpb1 >= 32);
-  if (!e.out_f32 && e.split_col >= N && aligned && gate_ok && make_store_map(mo, e.out, M, N, e.ldo) &&
-      (!e.hist_out || make_store_map(mh, e.hist_out, M, N, e.ldo)))
-    tm->staged = 1;
+  tm->staged = staged_maps(e, M, N, mo, mh) ? 1 : 0;
   return true;
 }
 }  // namespace
@@ -1106,11 +1381,12 @@ cudaError_t gemm_tc_grouped(int M0, const void* A0, const void* W0, const EpiArg
     const long long tiles = rows_t * ((N + bn - 1) / bn);
     const int grid = 2 * (int)(tiles < pairs ? tiles : pairs);
     const int ln = std::max(ln_side(e0), ln_side(e1));
+    const int epi = epi_form(e0) == EPI_PLAIN && epi_form(e1) == EPI_PLAIN ? EPI_PLAIN : EPI_FULL;
     if (bn == 256)
-      launch_pdl(gemm2_fn<256, true>(ln), grid, THREADS, Cfg2<256>::SMEM, s, a0, b0, o0, h0, M0, N, K, t0, e0, a1, b1, o1,
+      launch_pdl(gemm2_fn<256, true>(ln, epi), grid, THREADS, Cfg2<256>::SMEM, s, a0, b0, o0, h0, M0, N, K, t0, e0, a1, b1, o1,
                  h1, M1, t1, e1);
     else
-      launch_pdl(gemm2_fn<128, true>(ln), grid, THREADS, Cfg2<128>::SMEM, s, a0, b0, o0, h0, M0, N, K, t0, e0, a1, b1, o1,
+      launch_pdl(gemm2_fn<128, true>(ln, epi), grid, THREADS, Cfg2<128>::SMEM, s, a0, b0, o0, h0, M0, N, K, t0, e0, a1, b1, o1,
                  h1, M1, t1, e1);
     return launched();
   }
@@ -1130,7 +1406,8 @@ cudaError_t gemm_tc_grouped(int M0, const void* A0, const void* W0, const EpiArg
   const long long tiles = (long long)t0.n_tiles + t1.n_tiles;
   const int grid = (int)(tiles < g_sms ? tiles : g_sms);
   const int ln = std::max(ln_side(e0), ln_side(e1));
-  launch_pdl(gemm_fn<256, true>(ln), grid, THREADS, Cfg<256>::SMEM, s, a0, b0, a0, a0, o0, h0, a0, a0, M0, N, K, t0, e0, a1,
+  const int epi = epi_form(e0) == EPI_PLAIN && epi_form(e1) == EPI_PLAIN ? EPI_PLAIN : EPI_FULL;
+  launch_pdl(gemm_fn<256, true>(ln, epi), grid, THREADS, Cfg<256>::SMEM, s, a0, b0, a0, a0, o0, h0, a0, a0, M0, N, K, t0, e0, a1,
              b1, o1, h1, M1, t1, e1);
   return launched();
 }

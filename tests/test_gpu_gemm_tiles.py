@@ -51,3 +51,34 @@ def test_gemm_tiles(cuda, M, N, K, rpb, epilogue):
     if hist is not None:
         assert rel_l2(f64(hist)[:M], f64(out) - f64(base)) < 4e-3
         assert torch.all(hist[M] == 5.0)
+
+
+# one tile per CTA with a residual: normal and swapped tiles, blocks cut by M
+# and N, warps and blocks whose rows lie in two samples, bias and gate that are
+# not 16-byte aligned
+@pytest.mark.parametrize("M,N,K,rpb", [(4096, 1152, 200, 256), (1000, 1160, 64, 100), (300, 1288, 72, 33),
+                                       (130, 392, 1152, 130), (900, 904, 136, 900), (96, 264, 64, 32)])
+@pytest.mark.parametrize("epilogue", ["resid", "gelu_gated", "gated_history"])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_gemm_single_tile(cuda, M, N, K, rpb, epilogue, shift):
+    a, w = randn((M, K), "bf16", 1), randn((N, K), "bf16", 2, 0.1)
+    bias = randn(N + 8, "bf16", 3)[shift:shift + N]
+    resid = randn((M, N), "bf16", 8)
+    buf = torch.full((M + 1, N), 5.0, dtype=torch.bfloat16, device=cuda)
+    hist = torch.full((M + 1, N), 5.0, dtype=torch.bfloat16, device=cuda)
+    out, y, kw = buf[:M], f64(a) @ f64(w).T + f64(bias), {}
+    if epilogue != "resid":
+        gate = randn((-(-M // rpb), 2 * N + shift), "f32", 7)[:, N:2 * N]
+        kw = dict(gate=gate, gate_stride=2 * N + shift, rows_per_batch=rpb)
+        y = (oracle.model.gelu_tanh(y) if epilogue == "gelu_gated" else y) * f64(gate)[torch.arange(M).numpy() // rpb]
+    if epilogue == "gelu_gated":
+        kw["act"] = 1
+    if epilogue == "gated_history":
+        base = randn((M, N), "bf16", 9)
+        kw.update(hist_base=base, hist_out=hist[:M])
+    ff.featfix_op_gemm("bf16", a, w, out, bias=bias, resid=resid, **kw)
+    torch.cuda.synchronize()
+    assert rel_l2(f64(out), f64(resid) + y) < 4e-3
+    assert torch.all(buf[M] == 5.0) and torch.all(hist[M] == 5.0)
+    if epilogue == "gated_history":
+        assert rel_l2(f64(hist)[:M], f64(out) - f64(base)) < 4e-3
