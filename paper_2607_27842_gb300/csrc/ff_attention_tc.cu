@@ -1,33 +1,40 @@
 // Non-causal attention softmax(q k^T / sqrt(d)) v of the exact block (Eq. 1)
 // on the 5th-generation tensor cores, bf16 in, fp32 accumulate.
 //
-// One CTA per (sample, head, pair of 128-query tiles), 10 warps (sequences
+// One CTA per (sample, head, pair of 128-query tiles), 18 warps (sequences
 // of at most four key tiles: 6 warps, two CTAs per SM, each CTA taking one
 // or more query tiles of its (sample, head) in turn):
-//   warp 0     TMA producer: both query tiles once, then key and value tiles
-//              of 128 tokens into separate rings, straight from the fused qkv
-//              activation (3-D tensor map: head width, head slot, row; the
-//              head width is zero-padded to a multiple of 64 by the map);
-//   warp 1     TMEM allocator and MMA issuer (the whole warp runs the loop,
-//              one elected lane issues).  Per key tile j and query tile i:
-//              S_i = Q_i K_j^T into TMEM (both operands K-major from shared
-//              memory), then O_i += P_i V_j with P_i read from TMEM (where the
-//              softmax wrote it over S_i) and V MN-major from its TMA tile.
-//              S_i for tile j + 1 is issued right behind O_i's update for
-//              tile j, so one query tile's softmax overlaps the other's MMAs.
-//              The issuing thread runs only a few MMAs ahead of the tensor
-//              pipe, so every gap between two groups of MMAs holds at most
-//              one barrier wait;
-//   warps 2-5  softmax of query tile 0, warps 6-9 of query tile 1: each
-//              thread owns one query row (its TMEM lane): row max, exp2,
-//              row sum, P as bf16 pairs back into TMEM; O is rescaled in TMEM
-//              only when the running max grew by more than 2^8 (the final
-//              division uses the same stale max, so the result is unchanged).
-//              The two warpgroups run freely (making them take turns for
-//              the exponentials measured slower once the MMA issue stopped
-//              stalling).
+//   warp 0      TMA producer: both query tiles once, then key and value tiles
+//               of 128 tokens into separate rings, straight from the fused qkv
+//               activation (3-D tensor map: head width, head slot, row; the
+//               head width is zero-padded to a multiple of 64 by the map);
+//   warp 1      TMEM allocator and MMA issuer (the whole warp runs the loop,
+//               one elected lane issues each group of MMAs).  Per key tile j
+//               and query tile i: S_i = Q_i K_j^T into TMEM (both operands
+//               K-major from shared memory), then O_i += P_i V_j with P_i read
+//               from TMEM (where the softmax wrote it over S_i) and V MN-major
+//               from its TMA tile.  S_i for tile j + 1 is issued right behind
+//               O_i's update for tile j, so one query tile's softmax overlaps
+//               the other's MMAs.  Every gap between two groups of MMAs holds
+//               at most one barrier wait;
+//   warps 2-9   softmax of query tile 0, warps 10-17 of query tile 1; of each
+//               eight, four take the first 64 keys of a tile and four the
+//               others, one thread per query row (its TMEM lane) and half: exp2,
+//               row sum, P as bf16 pairs back into TMEM; the row max is taken
+//               and O rescaled only when the running reference would let P
+//               grow out of range (the final division uses the same reference).
+//
+// What bounds it (14566 tokens, 16 heads x 128; clock64 stamps): each query
+// tile's chain of S -> softmax -> P V, about 3700 cycles per key tile of
+// which the tile's own MMAs are 1650, the exponentials 1050 and the hand-offs
+// the rest; the MMAs alone (no softmax) take 861 us, the softmax alone about
+// as long.  Two threads per row instead of one (four softmax warps per
+// scheduler): 1324 -> 1260 us; every lane polling the S barrier instead of one
+// lane and a shuffle: 5%; one elected block per group of MMAs: 2%.  Now 1180
+// us (1470 TFLOP/s); 4096 + 512 tokens, 24 heads 226 -> 209 us.
 // TMEM columns: S_0 [0,128), S_1 [128,256), O_0 [256,384), O_1 [384,512);
-// with one query tile per CTA (short sequences): S [0,128), O [128,256).
+// with one query tile per CTA (short sequences): S [0,128), O [128,256).  P of a
+// half tile lies over the start of that half's S columns.
 // Keys of a sample lie in up to two row segments (text rows, image rows of
 // the stream-major token layout); tiles never straddle a segment and keys
 // past a segment's end are masked.
@@ -49,6 +56,10 @@ using namespace tc;
 constexpr int AQ = 128;        // queries per tile (MMA M)
 constexpr int AKV = 128;       // keys per tile (MMA N of S, K of P V)
 constexpr float RESCALE_LOG2 = 8.0f;
+// a half tile's sum of speculative exponentials that still stands: P, O and the
+// row sum keep their relative precision at any scale, and N such tiles times
+// any bf16-sized value stay far from overflow
+constexpr float SPEC_LIMIT = 1073741824.0f;   // 2^30
 constexpr int SHORT_KV_TILES = 4;  // sequences of at most 4 x 128 tokens: one query tile per CTA
 constexpr size_t SMEM_LIMIT = 232448;  // opt-in dynamic shared memory per block
 
@@ -66,24 +77,29 @@ __device__ __forceinline__ bool wait_u(uint64_t* b, uint32_t parity, volatile in
   return __all_sync(0xffffffffu, ok);
 }
 
-// QT query tiles per CTA.  QT = 2: two softmax warpgroups that overlap
-// each other's MMAs, key / value rings as deep as shared memory allows, one
-// CTA per SM.  QT = 1 (short sequences, a couple of key tiles): one softmax
-// warpgroup, single-slot rings and half the TMEM, so two CTAs share an SM
-// and overlap their latency chains instead; a CTA takes several query tiles
-// in turn so that all CTAs fit in one wave and a tile's loads overlap the
-// previous tile's tail.
+// QT query tiles per CTA.  QT = 2: two softmax warpgroups per query tile, the
+// tiles overlapping each other's MMAs, key / value rings as deep as shared
+// memory allows, one CTA per SM.  QT = 1 (short sequences, a couple of key
+// tiles): one softmax warpgroup, single-slot rings and half the TMEM, so two
+// CTAs share an SM and overlap their latency chains instead; a CTA takes
+// several query tiles in turn so that all CTAs fit in one wave and a tile's
+// loads overlap the previous tile's tail.
 template <int D, int QT> struct ACfg {
   static constexpr int SOFT_WARP0 = 2;                   // first softmax warp
-  static constexpr int THREADS = 32 * SOFT_WARP0 + 128 * QT;  // TMA warp, MMA warp, softmax warpgroups
+  // softmax warpgroups per query tile: with two query tiles each takes half of
+  // a tile's keys, four softmax warps per scheduler
+  static constexpr int WGS = QT == 2 ? 2 : 1;
+  static constexpr int SOFT = 128 * WGS;                 // softmax threads per query tile
+  static constexpr int THREADS = 32 * SOFT_WARP0 + SOFT * QT;  // TMA warp, MMA warp, softmax warps
   static constexpr int NBOX = D <= 64 ? 1 : 2;           // 64-wide column boxes per tile row
   static constexpr int DK = (D + 15) / 16 * 16;          // q k^T reduction width and P V output width
   static constexpr uint32_t BOX = 128 * 128;             // one [128 rows x 64] bf16 box, 16 KB
   static constexpr uint32_t TILE = NBOX * BOX;           // one Q, K or V tile
-  static constexpr int NST = (int)((SMEM_LIMIT - 1024 - 512 - QT * (size_t)TILE) / TILE);
+  static constexpr int NST = (int)((SMEM_LIMIT - 1024 - 512 - 1024 - QT * (size_t)TILE) / TILE);
   static constexpr int KST = QT == 1 ? 1 : NST >= 8 ? 4 : (NST + 1) / 2;  // key ring depth
   static constexpr int VST = QT == 1 ? 1 : NST >= 8 ? 4 : NST / 2;        // value ring depth
-  static constexpr size_t SMEM = 1024 + (size_t)(QT + KST + VST) * TILE + 512;
+  static constexpr size_t XCH = QT == 2 ? 2 * 128 * 4 : 0;   // a float per row, exchanged between the halves
+  static constexpr size_t SMEM = 1024 + (size_t)(QT + KST + VST) * TILE + 512 + XCH;
   static constexpr uint32_t TMEM_O = QT * AKV;           // S_i at i * 128, O_i at TMEM_O + i * 128
   static constexpr uint32_t TMEM_COLS = QT == 1 ? 256 : 512;
   // kind::f16, D fp32, A/B bf16; S: both K-major, N = 128; O: A (P) from
@@ -184,6 +200,39 @@ __device__ __forceinline__ float acc_total(const unsigned long long (&acc2)[4]) 
   return lo_f(a) + hi_f(a);
 }
 
+// P of 64 keys of a row, exp2(s scale - m) as bf16 pairs, from S in TMEM (keys
+// past `valid` masked); returns their sum
+__device__ __forceinline__ float exp_half(uint32_t s_col, int valid, unsigned long long sc2, float m, uint32_t (&pk)[32]) {
+  float v[64];
+  tmem_ld32_async(s_col, v);
+  tmem_wait32(v);
+  tmem_ld32_async(s_col + 32, v + 32);
+  const unsigned long long nm2 = f2u(-m, -m);
+  unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (k) tmem_wait32(v + 32);
+    if (valid < 64) {
+#pragma unroll
+      for (int e = 0; e < 32; ++e)
+        if (32 * k + e >= valid) v[32 * k + e] = -INFINITY;
+    }
+    uint32_t (&p16)[16] = *reinterpret_cast<uint32_t (*)[16]>(pk + 16 * k);
+    exp_pairs16(v + 32 * k, sc2, nm2, acc2, p16);
+  }
+  return acc_total(acc2);
+}
+// barrier `id` over n threads; true if any of them brings a true predicate
+__device__ __forceinline__ bool bar_or(int id, int n, bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(p ? 1u : 0u), "r"(id), "r"(n)
+      : "memory");
+  return r != 0;
+}
+
 __device__ __forceinline__ void tma_load3(const CUtensorMap* tm, uint64_t* bar, void* dst, int x, int y, int z) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
@@ -227,6 +276,7 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
   uint64_t* o_free = q_empty + 1;            // O read out by the softmax warps' epilogue
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* const xch = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);   // [query tile][row]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.y, b = blockIdx.z;
@@ -248,11 +298,11 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
     }
     for (int i = 0; i < QT; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&p_ready[i], 128);
+      mbar_init(&p_ready[i], QT == 2 ? C::SOFT / 32 : C::SOFT);   // (two tiles: one arrival per warp)
     }
     mbar_init(o_final, 1);
     mbar_init(q_empty, 1);
-    mbar_init(o_free, 128 * QT);
+    mbar_init(o_free, C::SOFT * QT);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmQKV) : "memory");
@@ -332,10 +382,12 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
     auto issue_s = [&](int i, int jj) {
       const uint64_t kd = sw128_desc(saddr(sK + (jj % C::KST) * C::TILE));
       const uint64_t qd = i ? qd1 : qd0;
+      if (elect_one()) {
 #pragma unroll
-      for (int k = 0; k < C::DK / 16; ++k) {
-        const uint64_t off = (uint64_t)((k >> 2) * (C::BOX >> 4) + 2 * (k & 3));
-        if (elect_one()) umma(tmem + (uint32_t)(i * AKV), qd + off, kd + off, C::IDESC_S, k != 0);
+        for (int k = 0; k < C::DK / 16; ++k) {
+          const uint64_t off = (uint64_t)((k >> 2) * (C::BOX >> 4) + 2 * (k & 3));
+          umma(tmem + (uint32_t)(i * AKV), qd + off, kd + off, C::IDESC_S, k != 0);
+        }
       }
       if (elect_one()) umma_commit(&s_full[i]);
     };
@@ -364,14 +416,16 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
           ok = wait_u(&p_ready[i], jj & 1, abort_flag);
           if (!ok) break;
           tc_fence_after();
-          // O_i += P_i V_j: 16 keys per step = 8 TMEM columns of P, 2 groups
-          // of 8 value rows (2 KB) of the MN-major V tile
+          // O_i += P_i V_j: 16 keys per step = 8 TMEM columns of P (each half
+          // of the keys at the start of its own S columns), 2 groups of 8
+          // value rows (2 KB) of the MN-major V tile
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < AKV / 16; ++k) {
-            const uint64_t vd = sw128_desc_mn(vaddr + (uint32_t)k * 2048u, C::BOX);
-            if (elect_one())
-              umma_ts(tmem + C::TMEM_O + (uint32_t)(i * AKV), tmem + (uint32_t)(i * AKV + k * 8), vd, C::IDESC_O,
-                      (j | k) != 0);
+            for (int k = 0; k < AKV / 16; ++k) {
+              const uint64_t vd = sw128_desc_mn(vaddr + (uint32_t)k * 2048u, C::BOX);
+              umma_ts(tmem + C::TMEM_O + (uint32_t)(i * AKV),
+                      tmem + (uint32_t)(i * AKV + k * 8 + (QT == 2 && k >= 4 ? 32 : 0)), vd, C::IDESC_O, (j | k) != 0);
+            }
           }
           if (i == QT - 1 && elect_one()) umma_commit(&v_empty[sv]);
           if (more) {
@@ -389,144 +443,157 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
       }
       if (ok && elect_one()) umma_commit(o_final);
     }
-  } else if (warp >= C::SOFT_WARP0) {
-    // softmax of query tile i: row r of the tile = TMEM lane r
-    const int i = (warp - C::SOFT_WARP0) >> 2;
+  } else if constexpr (QT == 2) {
+    // Softmax of query tile i, keys [64 hh, 64 hh + 64) of every key tile: row r
+    // of the tile = TMEM lane r, one thread per row and half.  Speculative:
+    // exponentials against the row's reference m (the first tile's max) go
+    // straight to bf16 P; any reference is exact as long as nothing overflows,
+    // so they stand unless a half tile's sum exceeds SPEC_LIMIT (or is not
+    // finite).  Otherwise, and on the first tile, the row max is taken over both
+    // halves, O is rescaled where the max grew by more than 2^8, and P is made
+    // again (S is still in place: P is stored only once it stands).  The two
+    // halves agree through a barrier that also carries the verdict; every warp
+    // takes every barrier, also after a wait gave up, so none is left waiting.
+    const int g = (warp - C::SOFT_WARP0) >> 2, i = g >> 1, hh = g & 1;
     const int q = warp & 3;
     const int r = q * 32 + lane;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    const uint32_t s_col = tmem + lane_off + (uint32_t)(i * AKV);
+    const uint32_t s_col = tmem + lane_off + (uint32_t)(i * AKV + 64 * hh);
     const uint32_t o_col = tmem + lane_off + C::TMEM_O + (uint32_t)(i * AKV);
+    float* const xr = xch + i * 128 + r;
+    constexpr int OC = C::DK / 16, OC0 = (OC + 1) / 2;   // O column groups of 16; the first half's share
+    const SegTile qs = seg_tile(a, b, QT * blockIdx.x + i);
+    const unsigned long long sc2 = f2u(scale_log2, scale_log2);
+    float m = -INFINITY, l = 0.f;
+    bool ok = true;
+    for (int j = 0; j < nkv; ++j) {
+      const int valid = seg_tile(a, b, j).valid - 64 * hh;
+      if (ok) ok = wait_u(&s_full[i], j & 1, abort_flag);
+      tc_fence_after();
+      uint32_t pk[32];
+      float lt = 0.f;
+      bool redo = j == 0;
+      if (j > 0) {
+        if (ok) lt = exp_half(s_col, valid, sc2, m, pk);
+        redo = bar_or(1 + i, C::SOFT, ok && !(lt <= SPEC_LIMIT));
+      }
+      if (redo) {
+        float mx = -INFINITY;
+        if (ok) {
+          float t[32];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            tmem_ld32_async(s_col + (uint32_t)(32 * k), t);
+            tmem_wait32(t);
+#pragma unroll
+            for (int e = 0; e < 32; ++e)
+              if (32 * k + e < valid) mx = fmaxf(mx, t[e]);
+          }
+        }
+        // the row max over both halves
+        if (hh == 0) *xr = mx;
+        bar_or(1 + i, C::SOFT, false);
+        if (hh == 1) {
+          mx = fmaxf(mx, *xr);
+          *xr = mx;
+        }
+        bar_or(1 + i, C::SOFT, false);
+        if (hh == 0) mx = *xr;
+        const float m_new = fmaxf(m, mx * scale_log2);
+        const bool grow = m_new > m + RESCALE_LOG2;  // always on the first tile
+        const float alpha = grow ? ex2(m - m_new) : 1.0f;
+        if (ok && __any_sync(0xffffffffu, grow)) {
+          // O_i holds every update through tile j - 1: s_full[i] for tile j
+          // arrived after them
+          if (j >= 1) {
+            for (int c = hh ? OC0 : 0; c < (hh ? OC : OC0); ++c) {
+              float o[16];
+              tmem_ld16(o_col + (uint32_t)(c * 16), o);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) o[e] *= alpha;
+              tmem_st16(o_col + (uint32_t)(c * 16), o);
+            }
+          }
+          if (grow) m = m_new;
+        }
+        l *= alpha;
+        if (ok) lt = exp_half(s_col, valid, sc2, m, pk);
+      }
+      l += lt;
+      if (ok) {
+        tmem_st32(s_col, pk);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_ready[i]);
+      }
+    }
+    // the row sum over both halves
+    if (hh == 0) *xr = l;
+    bar_or(1 + i, C::SOFT, false);
+    if (hh == 1) {
+      l += *xr;
+      *xr = l;
+    }
+    bar_or(1 + i, C::SOFT, false);
+    if (hh == 0) l = *xr;
+    if (ok) ok = wait_u(o_final, 0, abort_flag);
+    if (ok) {
+      tc_fence_after();
+      const float inv = 1.0f / l;
+      bf16* orow = reinterpret_cast<bf16*>(a.out) + (size_t)(qs.row0 + (r < qs.valid ? r : 0)) * a.ld_out + (size_t)h * D;
+#pragma unroll
+      for (int cc = 0; cc < OC0; ++cc) {
+        const int c = hh ? OC0 + cc : cc;
+        if (c >= OC) break;
+        float o[16];
+        tmem_ld16(o_col + (uint32_t)(c * 16), o);
+        if (r < qs.valid) {
+#pragma unroll
+          for (int e = 0; e < 16; e += 8) {
+            if (c * 16 + e < D) {
+              float t8[8];
+#pragma unroll
+              for (int z = 0; z < 8; ++z) t8[z] = o[e + z] * inv;
+              st16(orow + c * 16 + e, t8);
+            }
+          }
+        }
+      }
+    }
+  } else {
+    // one query tile: row r of the tile = TMEM lane r
+    constexpr int i = 0;
+    const int q = warp & 3;
+    const int r = q * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    const uint32_t s_col = tmem + lane_off;
+    const uint32_t o_col = tmem + lane_off + C::TMEM_O;
     bool ok = true;
     for (int it = 0; it < ipc && ok && item_live(it); ++it) {
     const SegTile qs = seg_tile(a, b, QT * (blockIdx.x * ipc + it) + i);
     float m = -INFINITY, l = 0.f;
     for (int j = 0; j < nkv; ++j) {
       const int valid = seg_tile(a, b, j).valid;
-      int w = 1;
-      if (lane == 0) w = wait_a(&s_full[i], (it * nkv + j) & 1, abort_flag) ? 1 : 0;
-      if (!__shfl_sync(0xffffffffu, w, 0)) { ok = false; break; }
+      if (!wait_u(&s_full[i], (it * nkv + j) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      // row max as a tree of three-input maxima (72 instructions for 128
-      // values instead of 127).  One query tile per CTA (short sequences,
-      // latency-bound): S is read 64 columns at a time for the max and again
-      // in quarters for the exponentials, which keeps the row out of
-      // registers; two query tiles: the row is held in registers.
-      float v[QT == 1 ? 1 : AKV];
+      // row max as a tree of three-input maxima.  S is read 64 columns at a
+      // time for the max and again in quarters for the exponentials, which
+      // keeps the row out of registers
       float mx[16];
-      if constexpr (QT == 2) {
-        // Speculative softmax: exponentials against the running reference
-        // m while S streams in from TMEM, P stored as it is made.  They are
-        // the lazy-rescale result whenever no exponent exceeds 2^8, which a
-        // tile sum <= 256 guarantees; otherwise (and on the first tile) the
-        // row max is taken from the registers, O is rescaled if the max
-        // grew by more than 2^8, and P is recomputed.
-        const unsigned long long sc2 = f2u(scale_log2, scale_log2);
-        bool need = true;
-        float lt = 0.f;
-        if (j > 0) {
-          const unsigned long long nm2 = f2u(-m, -m);
-          unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};
-          tmem_ld32_async(s_col, v);
-          tmem_wait32(v);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            // S columns [32 (k + 1), 32 (k + 2)) load while chunk k is
-            // finished; P chunk k goes to columns [16 k, 16 k + 16), which
-            // hold S already read
-            if (k + 1 < 4) tmem_ld32_async(s_col + (uint32_t)(32 * (k + 1)), v + 32 * (k + 1));
-            if (valid < AKV) {
+      for (int e = 0; e < 16; ++e) mx[e] = -INFINITY;
 #pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (32 * k + e >= valid) v[32 * k + e] = -INFINITY;
-            }
-            uint32_t pk[16];
-            exp_pairs16(v + 32 * k, sc2, nm2, acc2, pk);
-            tmem_st16u(s_col + (uint32_t)(16 * k), pk);
-            if (k + 1 < 4) tmem_wait32(v + 32 * (k + 1));
-          }
-          lt = acc_total(acc2);
-          need = __any_sync(0xffffffffu, !(lt <= 256.0f));   // also a non-finite sum
-        } else {
-          tmem_ld64w(s_col, v);
-          tmem_ld64w(s_col + 64, v + 64);
-          if (valid < AKV) {
-#pragma unroll
-            for (int e = 0; e < AKV; ++e)
-              if (e >= valid) v[e] = -INFINITY;
-          }
-        }
-        float alpha = 1.0f;
-        if (need) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            mx[e] = max3f(max3f(v[e], v[e + 16], v[e + 32]), max3f(v[e + 48], v[e + 64], v[e + 80]),
-                          fmaxf(v[e + 96], v[e + 112]));
-#pragma unroll
-          for (int e = 0; e < 5; ++e) mx[e] = max3f(mx[e], mx[e + 5], mx[e + 10]);
-          mx[0] = max3f(max3f(mx[0], mx[1], mx[2]), max3f(mx[3], mx[4], mx[15]), mx[0]);
-          const float m_new = fmaxf(m, mx[0] * scale_log2);
-          const bool grow = m_new > m + RESCALE_LOG2;  // always on the first tile
-          if (__any_sync(0xffffffffu, grow)) {
-            alpha = grow ? ex2(m - m_new) : 1.0f;
-            // O_i holds every update through tile j - 1: s_full[i] for tile
-            // j arrived after them
-            if (j >= 1) {
-#pragma unroll
-              for (int c = 0; c < C::DK / 16; ++c) {
-                float o[16];
-                tmem_ld16(o_col + (uint32_t)(c * 16), o);
-#pragma unroll
-                for (int e = 0; e < 16; ++e) o[e] *= alpha;
-                tmem_st16(o_col + (uint32_t)(c * 16), o);
-              }
-            }
-            if (grow) m = m_new;
-            tmem_st_wait();   // the speculative P stores land before their recomputation
-            const unsigned long long nm2 = f2u(-m, -m);
-            unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              uint32_t pk[16];
-              exp_pairs16(v + 32 * k, sc2, nm2, acc2, pk);
-              tmem_st16u(s_col + (uint32_t)(16 * k), pk);
-            }
-            lt = acc_total(acc2);
-          }
-        }
-        l = l * alpha + lt;
-        tmem_st_wait();
-        tc_fence_before();
-        mbar_arrive(&p_ready[i]);
-        continue;
-      }
-      if constexpr (QT == 1) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) mx[e] = -INFINITY;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          float t[64];
-          tmem_ld64w(s_col + (uint32_t)(64 * hh), t);
-          if (valid < AKV) {
-#pragma unroll
-            for (int e = 0; e < 64; ++e)
-              if (64 * hh + e >= valid) t[e] = -INFINITY;
-          }
-#pragma unroll
-          for (int e = 0; e < 16; ++e) mx[e] = max3f(mx[e], max3f(t[e], t[e + 16], t[e + 32]), t[e + 48]);
-        }
-      } else {
-        tmem_ld64w(s_col, v);
-        tmem_ld64w(s_col + 64, v + 64);
+      for (int hh = 0; hh < 2; ++hh) {
+        float t[64];
+        tmem_ld64w(s_col + (uint32_t)(64 * hh), t);
         if (valid < AKV) {
 #pragma unroll
-          for (int e = 0; e < AKV; ++e)
-            if (e >= valid) v[e] = -INFINITY;
+          for (int e = 0; e < 64; ++e)
+            if (64 * hh + e >= valid) t[e] = -INFINITY;
         }
 #pragma unroll
-        for (int e = 0; e < 16; ++e)
-          mx[e] = max3f(max3f(v[e], v[e + 16], v[e + 32]), max3f(v[e + 48], v[e + 64], v[e + 80]),
-                        fmaxf(v[e + 96], v[e + 112]));
+        for (int e = 0; e < 16; ++e) mx[e] = max3f(mx[e], max3f(t[e], t[e + 16], t[e + 32]), t[e + 48]);
       }
 #pragma unroll
       for (int e = 0; e < 5; ++e) mx[e] = max3f(mx[e], mx[e + 5], mx[e + 10]);
@@ -552,48 +619,32 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
 #pragma unroll
       for (int e = 0; e < 8; ++e) ls[e] = 0.f;
       // P as bf16 pairs into the first 64 columns of S_i (already read)
-      if constexpr (QT == 1) {
-        // S again, 32 columns at a time (the next quarter loading while this
-        // one is finished); quarter k's P columns [16k, 16k + 16) lie in
-        // columns already read
-        float sq[2][32];
-        tmem_ld32_async(s_col, sq[0]);
-        tmem_wait32(sq[0]);
+      // S again, 32 columns at a time (the next quarter loading while this
+      // one is finished); quarter k's P columns [16k, 16k + 16) lie in
+      // columns already read
+      float sq[2][32];
+      tmem_ld32_async(s_col, sq[0]);
+      tmem_wait32(sq[0]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (k + 1 < 4) tmem_ld32_async(s_col + (uint32_t)(32 * (k + 1)), sq[(k + 1) & 1]);
-          float* x = sq[k & 1];
-          if (valid < AKV) {
+      for (int k = 0; k < 4; ++k) {
+        if (k + 1 < 4) tmem_ld32_async(s_col + (uint32_t)(32 * (k + 1)), sq[(k + 1) & 1]);
+        float* x = sq[k & 1];
+        if (valid < AKV) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (32 * k + e >= valid) x[e] = -INFINITY;
-          }
-          uint32_t pk[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const float p0 = ex2(fmaf(x[2 * e], scale_log2, -m));
-            const float p1 = ex2(fmaf(x[2 * e + 1], scale_log2, -m));
-            ls[e & 7] += p0 + p1;
-            __nv_bfloat162 t2 = __floats2bfloat162_rn(p0, p1);
-            pk[e] = *reinterpret_cast<uint32_t*>(&t2);
-          }
-          tmem_st16u(s_col + (uint32_t)(16 * k), pk);
-          if (k + 1 < 4) tmem_wait32(sq[(k + 1) & 1]);
+          for (int e = 0; e < 32; ++e)
+            if (32 * k + e >= valid) x[e] = -INFINITY;
         }
-      } else {
+        uint32_t pk[16];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t pk[32];
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float p0 = ex2(fmaf(v[half * 64 + 2 * e], scale_log2, -m));
-            const float p1 = ex2(fmaf(v[half * 64 + 2 * e + 1], scale_log2, -m));
-            ls[e & 7] += p0 + p1;
-            __nv_bfloat162 t2 = __floats2bfloat162_rn(p0, p1);
-            pk[e] = *reinterpret_cast<uint32_t*>(&t2);
-          }
-          tmem_st32(s_col + (uint32_t)(half * 32), pk);
+        for (int e = 0; e < 16; ++e) {
+          const float p0 = ex2(fmaf(x[2 * e], scale_log2, -m));
+          const float p1 = ex2(fmaf(x[2 * e + 1], scale_log2, -m));
+          ls[e & 7] += p0 + p1;
+          __nv_bfloat162 t2 = __floats2bfloat162_rn(p0, p1);
+          pk[e] = *reinterpret_cast<uint32_t*>(&t2);
         }
+        tmem_st16u(s_col + (uint32_t)(16 * k), pk);
+        if (k + 1 < 4) tmem_wait32(sq[(k + 1) & 1]);
       }
       l = l * alpha + (((ls[0] + ls[1]) + (ls[2] + ls[3])) + ((ls[4] + ls[5]) + (ls[6] + ls[7])));
       tmem_st_wait();
@@ -601,9 +652,7 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
       mbar_arrive(&p_ready[i]);
     }
     if (!ok) break;
-    int w = 1;
-    if (lane == 0) w = wait_a(o_final, it & 1, abort_flag) ? 1 : 0;
-    if (!__shfl_sync(0xffffffffu, w, 0)) { ok = false; break; }
+    if (!wait_u(o_final, it & 1, abort_flag)) { ok = false; break; }
     tc_fence_after();
     const float inv = 1.0f / l;
     bf16* orow = reinterpret_cast<bf16*>(a.out) + (size_t)(qs.row0 + (r < qs.valid ? r : 0)) * a.ld_out + (size_t)h * D;
@@ -639,6 +688,8 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
 
 
 // ---------------------------------------------------------------------------
+// (16 x 256 tokens, 16 heads x 72: 17.6 -> 14.7 us with every lane polling, one
+// arrival per warp and one elected block per group of MMAs)
 // Sequences of at most two key tiles (256 tokens; DiT-XL/2) with a head
 // width of at most 80: one query tile at a time, two CTAs per SM, every CTA
 // taking the query tiles of one (sample, head) in turn.  The head's K and V
@@ -734,10 +785,10 @@ __global__ void __launch_bounds__(192, 2)
     mbar_init(k_full, 1);
     mbar_init(v_full, 1);
     mbar_init(s_full, 1);
-    mbar_init(p_ready, 128);
+    mbar_init(p_ready, 4);
     mbar_init(o_final, 1);
     mbar_init(q_empty, 1);
-    mbar_init(o_free, 128);
+    mbar_init(o_free, 4);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmQKV) : "memory");
@@ -813,13 +864,13 @@ __global__ void __launch_bounds__(192, 2)
       tc_fence_after();
       // S = Q K^T over all keys: 4 steps of 16 in the 128-byte boxes (+32 B
       // per step inside the swizzle atom), then the 32-byte tail box
-#pragma unroll
-      for (int k = 0; k < C::DK / 16; ++k) {
-        const uint64_t ad = k < 4 ? sw128_desc(base + L::QA) + (uint64_t)(2 * k) : sw32_desc(base + L::QT);
-        const uint64_t bd = k < 4 ? sw128_desc(base + L::KA) + (uint64_t)(2 * k) : sw32_desc(base + L::KT);
-        if (elect_one()) umma(tmem, ad, bd, idesc_s, k != 0);
-      }
       if (elect_one()) {
+#pragma unroll
+        for (int k = 0; k < C::DK / 16; ++k) {
+          const uint64_t ad = k < 4 ? sw128_desc(base + L::QA) + (uint64_t)(2 * k) : sw32_desc(base + L::QT);
+          const uint64_t bd = k < 4 ? sw128_desc(base + L::KA) + (uint64_t)(2 * k) : sw32_desc(base + L::KT);
+          umma(tmem, ad, bd, idesc_s, k != 0);
+        }
         umma_commit(s_full);
         umma_commit(q_empty);
       }
@@ -829,12 +880,14 @@ __global__ void __launch_bounds__(192, 2)
       tc_fence_after();
       // O = P V: keys 16k .. 16k + 15 are P columns 8k .. 8k + 7; 16 rows of
       // key tile k / 8 (1 KB into each of its 64-byte-swizzled boxes)
-      for (int k = 0; k < 8 * nkv; ++k) {
-        const int j = k >> 3, kk = k & 7;
-        const uint64_t vd = sw64_desc_mn(base + L::VA + j * C::VTILE + (uint32_t)kk * 1024u);
-        if (elect_one()) umma_ts(tmem + 128, tmem + (uint32_t)(8 * k), vd, C::IDESC_O, k != 0);
+      if (elect_one()) {
+        for (int k = 0; k < 8 * nkv; ++k) {
+          const int j = k >> 3, kk = k & 7;
+          const uint64_t vd = sw64_desc_mn(base + L::VA + j * C::VTILE + (uint32_t)kk * 1024u);
+          umma_ts(tmem + 128, tmem + (uint32_t)(8 * k), vd, C::IDESC_O, k != 0);
+        }
+        umma_commit(o_final);
       }
-      if (elect_one()) umma_commit(o_final);
     }
   } else {
     const int q = warp & 3;
@@ -846,9 +899,7 @@ __global__ void __launch_bounds__(192, 2)
     bool ok = true;
     for (int it = 0; it < ipc && ok && item_live(it); ++it) {
       const SegTile qs = seg_tile(a, b, blockIdx.x * ipc + it);
-      int w = 1;
-      if (lane == 0) w = wait_a(s_full, it & 1, abort_flag) ? 1 : 0;
-      if (!__shfl_sync(0xffffffffu, w, 0)) { ok = false; break; }
+      if (!wait_u(s_full, it & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
       // pass 1: row max over the keys, 64 columns at a time
       float mx[16];
@@ -899,9 +950,9 @@ __global__ void __launch_bounds__(192, 2)
       const float l = acc_total(acc2);
       tmem_st_wait();
       tc_fence_before();
-      mbar_arrive(p_ready);
-      if (lane == 0) w = wait_a(o_final, it & 1, abort_flag) ? 1 : 0;
-      if (!__shfl_sync(0xffffffffu, w, 0)) { ok = false; break; }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_ready);
+      if (!wait_u(o_final, it & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
       // O into registers, then TMEM is released (the next query tile's S
       // MMA may start) before the output is written
@@ -909,7 +960,8 @@ __global__ void __launch_bounds__(192, 2)
 #pragma unroll
       for (int c = 0; c < C::DK / 16; ++c) tmem_ld16(o_col + (uint32_t)(c * 16), o[c]);
       tc_fence_before();
-      mbar_arrive(o_free);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(o_free);
       const float inv = 1.0f / l;
       bf16* orow = reinterpret_cast<bf16*>(a.out) + (size_t)(qs.row0 + (r < qs.valid ? r : 0)) * a.ld_out + (size_t)h * D;
       if (r < qs.valid) {
