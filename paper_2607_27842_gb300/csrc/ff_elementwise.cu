@@ -6,7 +6,9 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 namespace cg = cooperative_groups;
 
@@ -468,8 +470,8 @@ cudaError_t launch_ln_ab(DType dt, const float* mod, long long mod_stride, int r
 
 // ---------------------------------------------------------------------------
 // adaLN branch input: LN(x) (no affine, eps 1e-6) * (1 + scale_b) + shift_b.
-// One warp per row, the row held in registers (NCH 16-byte vectors per
-// lane): one global read, exact two-pass mean / variance, one write.
+// One warp per row, exact two-pass mean / variance from registers, one global
+// read and one write.
 // ---------------------------------------------------------------------------
 // One warp per row (8 rows per block, for row counts that fill about two
 // waves at most); the block first stages the shift /
@@ -550,133 +552,239 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : 1) k_ln_mod1(const T* __re
   }
 }
 
-// Each warp takes rpw rows (8 warps, a block of 8 * rpw consecutive rows);
-// the block first stages the shift / scale vectors of its first row's
-// sample in shared memory (coalesced, read back by every warp of that sample
-// instead of 4 x 16 B per lane per chunk from global memory); a warp loads
-// its next row while it reduces and writes the current one.
-template <class T, int NCH>
-__global__ void __launch_bounds__(256) k_ln_mod(const T* __restrict__ x, T* __restrict__ out, long long rows, int C,
-                                                const float* __restrict__ shift, const float* __restrict__ scale,
-                                                int mod_stride, int seg_split, int rpb0, int rpb1, int rpw) {
+// Large row counts and wide rows: a block takes 8 * rpw consecutive rows, a warp
+// rpw of them in turn.  Rows reach the warp through its own ring of DEPTH slots in
+// shared memory by cp.async (each lane copies and reads back its own vectors,
+// so a row needs no barrier), so DEPTH rows per warp are in flight while one is
+// reduced; the shift / scale of the block's first sample (read back by every
+// warp of that sample) are copied the same way behind the first rows, so the
+// two latencies overlap.  Bound by latency and bytes in flight, not by
+// arithmetic (packed fp32 pairs changed nothing at 14310 x 2048).  Against rows
+// held a register row ahead: 8704 x 3072 38.6 -> 25.7 us, 4608 x 3072 24.4 ->
+// 18.8, 8192 x 1152 16.9 -> 12.7, 14000 x 128 10.3 -> 4.9, 14310 x 2048 24.4 ->
+// 24.1.
+__device__ __forceinline__ void cp16_async(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait_group() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// packed fp32 pairs (fma.rn.f32x2: two results an instruction)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2f(float a, float b) {
+  return (f32x2)__float_as_uint(a) | ((f32x2)__float_as_uint(b) << 32);
+}
+__device__ __forceinline__ float lo2(f32x2 x) { return __uint_as_float((unsigned)x); }
+__device__ __forceinline__ float hi2(f32x2 x) { return __uint_as_float((unsigned)(x >> 32)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// a 16-byte vector of four fp32 or eight bf16 values <-> pairs
+__device__ __forceinline__ void unpack2x(const uint4& v, f32x2 (&p)[2]) {
+  p[0] = (f32x2)v.x | ((f32x2)v.y << 32);
+  p[1] = (f32x2)v.z | ((f32x2)v.w << 32);
+}
+__device__ __forceinline__ void unpack2x(const uint4& v, f32x2 (&p)[4]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) p[i] = (f32x2)(w[i] << 16) | ((f32x2)(w[i] & 0xffff0000u) << 32);
+}
+__device__ __forceinline__ uint4 packv(const f32x2 (&o)[2]) {
+  return make_uint4((unsigned)o[0], (unsigned)(o[0] >> 32), (unsigned)o[1], (unsigned)(o[1] >> 32));
+}
+__device__ __forceinline__ uint4 packv(const f32x2 (&o)[4]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo2(o[i]), hi2(o[i]));
+    w[i] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+template <class T, int NCH, int DEPTH>
+__global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
+    k_ln_mod(const T* __restrict__ x, T* __restrict__ out, long long rows, int C, const float* __restrict__ shift,
+             const float* __restrict__ scale, int mod_stride, int seg_split, int rpb0, int rpb1, int rpw) {
   pdl_trigger();
   pdl_wait();
-  extern __shared__ float4 smod4[];                  // [2 * C / 4]: shift, then scale
+  extern __shared__ float4 smod4[];                  // [2 * C / 4]: shift, then scale; then the rings
   float* smod = reinterpret_cast<float*>(smod4);
   constexpr int V = VecN<T>::n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long r0 = (long long)blockIdx.x * 8 * rpw;
   const int b0 = (int)(r0 < seg_split ? r0 / rpb0 : (r0 - seg_split) / rpb1);
   const int nv = C / V;
-  // rows r0 + warp * rpw + t, t < rpw; the first one's loads go out before
-  // the staging
   const long long rw = r0 + (long long)warp * rpw;
-  uint4 cur[NCH];
-  auto load_row = [&](long long r, uint4 (&v)[NCH]) {
-    const T* xr = x + r * C;
+  const int n = (int)min((long long)rpw, rows - rw);  // the warp's rows (may be <= 0)
+  uint4* const ring = reinterpret_cast<uint4*>(smod4 + C / 2) + (size_t)warp * DEPTH * nv;
+  auto copy_row = [&](int t) {
+    const uint4* xr = reinterpret_cast<const uint4*>(x + (rw + t) * C);
+    uint4* d = ring + (t % DEPTH) * nv;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
       const int k = lane + 32 * j;
-      if (k < nv) v[j] = *reinterpret_cast<const uint4*>(xr + k * V);
+      if (k < nv) cp16_async(d + k, xr + k);
     }
   };
-  if (rw < rows) load_row(rw, cur);
-  {
-    const float4* sh4 = reinterpret_cast<const float4*>(shift + (size_t)b0 * mod_stride);
-    const float4* sc4 = reinterpret_cast<const float4*>(scale + (size_t)b0 * mod_stride);
-    for (int i = threadIdx.x; i < C / 4; i += blockDim.x) {
-      smod4[i] = sh4[i];
-      smod4[C / 4 + i] = sc4[i];
+#pragma unroll
+  for (int t = 0; t < DEPTH; ++t) {
+    if (t < n) copy_row(t);
+    if (t == 0) {
+      const float4* sh4 = reinterpret_cast<const float4*>(shift + (size_t)b0 * mod_stride);
+      const float4* sc4 = reinterpret_cast<const float4*>(scale + (size_t)b0 * mod_stride);
+      for (int i = threadIdx.x; i < C / 4; i += blockDim.x) {
+        cp16_async(smod4 + i, sh4 + i);
+        cp16_async(smod4 + C / 4 + i, sc4 + i);
+      }
     }
+    cp_commit_group();
+  }
+  cp_wait_group<DEPTH - 1>();
+  for (int i = threadIdx.x; i < C / 4; i += blockDim.x) {   // 1 + scale, each thread its own copies
+    float4 v = smod4[C / 4 + i];
+    v.x += 1.0f; v.y += 1.0f; v.z += 1.0f; v.w += 1.0f;
+    smod4[C / 4 + i] = v;
   }
   __syncthreads();
-  for (int t = 0; t < rpw; ++t) {
+  for (int t = 0; t < n; ++t) {
+    if (t > 0) cp_wait_group<DEPTH - 1>();
     const long long r = rw + t;
-    if (r >= rows) break;
-    uint4 nxt[NCH];
-    const bool more = t + 1 < rpw && r + 1 < rows;
-    if (more) load_row(r + 1, nxt);
-    float s = 0.f;
+    // the row as packed fp32 pairs where they fit the registers, else as stored
+    // (unpacked again in each pass)
+    constexpr bool KEEP = NCH * V <= 32;
+    uint4 cur[KEEP ? 1 : NCH];
+    f32x2 a[KEEP ? NCH : 1][V / 2];
+    const uint4* const slot = ring + (t % DEPTH) * nv;
+    f32x2 s2 = 0ull;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
       if (lane + 32 * j < nv) {
-        float a[V];
-        unpack16(cur[j], a);
+        const uint4 v = slot[lane + 32 * j];
+        if constexpr (!KEEP) cur[j] = v;
+        f32x2 (&p)[V / 2] = a[KEEP ? j : 0];
+        unpack2x(v, p);
 #pragma unroll
-        for (int q = 0; q < V; ++q) s += a[q];
+        for (int q = 0; q < V / 2; ++q) s2 = add2(s2, p[q]);
       }
     }
-    s = warp_sum(s);
-    const float mean = s / C;
-    float ss = 0.f;
+    const float mean = warp_sum(lo2(s2) + hi2(s2)) / C;
+    if (t + DEPTH < n) copy_row(t + DEPTH);          // the slot has been read (its values are in the sum)
+    cp_commit_group();
+    const f32x2 nm = pack2f(-mean, -mean);
+    f32x2 ss2 = 0ull;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
       if (lane + 32 * j < nv) {
-        float a[V];
-        unpack16(cur[j], a);
+        f32x2 (&p)[V / 2] = a[KEEP ? j : 0];
+        if constexpr (!KEEP) unpack2x(cur[j], p);
 #pragma unroll
-        for (int q = 0; q < V; ++q) { const float d = a[q] - mean; ss += d * d; }
-      }
-    }
-    ss = warp_sum(ss);
-    const float rstd = rsqrtf(ss / C + 1e-6f);
-    const int b = (int)(r < seg_split ? r / rpb0 : (r - seg_split) / rpb1);
-    // the block's sample from shared memory, another sample (a block
-    // straddling a sample boundary) from global memory
-    const float* sh = b == b0 ? smod : shift + (size_t)b * mod_stride;
-    const float* sc = b == b0 ? smod + C : scale + (size_t)b * mod_stride;
-    T* orow = out + r * C;
-#pragma unroll
-    for (int j = 0; j < NCH; ++j) {
-      const int k = lane + 32 * j;
-      if (k < nv) {
-        float a[V], o[V];
-        unpack16(cur[j], a);
-#pragma unroll
-        for (int q = 0; q < V; q += 4) {
-          const float4 s4 = *reinterpret_cast<const float4*>(sh + k * V + q);
-          const float4 c4 = *reinterpret_cast<const float4*>(sc + k * V + q);
-          o[q] = (a[q] - mean) * rstd * (1.0f + c4.x) + s4.x;
-          o[q + 1] = (a[q + 1] - mean) * rstd * (1.0f + c4.y) + s4.y;
-          o[q + 2] = (a[q + 2] - mean) * rstd * (1.0f + c4.z) + s4.z;
-          o[q + 3] = (a[q + 3] - mean) * rstd * (1.0f + c4.w) + s4.w;
+        for (int q = 0; q < V / 2; ++q) {
+          const f32x2 d = add2(p[q], nm);
+          if constexpr (KEEP) p[q] = d;              // centred from here on
+          ss2 = fma2(d, d, ss2);
         }
-        st16(orow + k * V, o);
       }
     }
-    if (more) {
+    const float rstd = rsqrtf(warp_sum(lo2(ss2) + hi2(ss2)) / C + 1e-6f);
+    const f32x2 rs = pack2f(rstd, rstd);
+    const int b = (int)(r < seg_split ? r / rpb0 : (r - seg_split) / rpb1);
+    uint4* const orow = reinterpret_cast<uint4*>(out + r * C);
+    // the block's sample from shared memory (scale already 1 + scale), another
+    // sample (a block straddling a sample boundary) from global memory
+    auto apply = [&](auto own, const float* sh, const float* sc) {
 #pragma unroll
-      for (int j = 0; j < NCH; ++j) cur[j] = nxt[j];
+      for (int j = 0; j < NCH; ++j) {
+        const int k = lane + 32 * j;
+        if (k < nv) {
+          f32x2 (&p)[V / 2] = a[KEEP ? j : 0];
+          if constexpr (!KEEP) unpack2x(cur[j], p);
+          f32x2 o[V / 2];
+#pragma unroll
+          for (int q = 0; q < V / 2; q += 2) {
+            const ulonglong2 s4 = *reinterpret_cast<const ulonglong2*>(sh + k * V + 2 * q);
+            ulonglong2 c4 = *reinterpret_cast<const ulonglong2*>(sc + k * V + 2 * q);
+            if constexpr (!decltype(own)::value) {
+              const f32x2 one = pack2f(1.0f, 1.0f);
+              c4.x = add2(c4.x, one);
+              c4.y = add2(c4.y, one);
+            }
+            o[q] = fma2(mul2(KEEP ? p[q] : add2(p[q], nm), rs), c4.x, s4.x);
+            o[q + 1] = fma2(mul2(KEEP ? p[q + 1] : add2(p[q + 1], nm), rs), c4.y, s4.y);
+          }
+          orow[k] = packv(o);
+        }
+      }
+    };
+    if (b == b0) apply(std::true_type{}, smod, smod + C);
+    else apply(std::false_type{}, shift + (size_t)b * mod_stride, scale + (size_t)b * mod_stride);
+  }
+}
+
+template <class T, int NCH>
+static cudaError_t ln_mod_launch(const T* x, T* out, long long rows, int C, const float* shift, const float* scale,
+                                 int mod_stride, int seg_split, int rpb0, int rpb1, cudaStream_t s) {
+  const long long sms = num_sms(), mods = 2LL * C * 4, row = (long long)C * sizeof(T);
+  // Rows of up to eight vectors per lane, while a row per warp makes at most
+  // about two waves of two blocks per SM: every row's loads in flight at once
+  // (64 x 128 fp32 1.93 us against 2.08 through the ring).
+  const bool few = rows <= 8LL * 4 * sms;
+  if constexpr (NCH <= 8) {
+    if (few) {
+      launch_pdl(k_ln_mod1<T, NCH>, (unsigned)((rows + 7) / 8), 256, (size_t)mods, s, x, out, rows, C, shift, scale,
+                 mod_stride, seg_split, rpb0, rpb1);
+      return launched();
     }
   }
+  // Blocks per SM as measured (8192 x 1152: four 12.7 us, two 16.6; 14310 x 2048:
+  // three 24.2, two 27.1, four 29.5; 8704 x 3072: two 25.7, three 33.5; 8000 x
+  // 2048 fp32: four 28.0, two 36.8), the ring as deep as their shared memory allows.
+  constexpr int BLOCKS = NCH <= 6 ? 4 : NCH <= 8 ? 3 : NCH <= 12 ? 2 : 4;
+  int rpw = 1, depth = 1;
+  if (!few) {
+    const long long budget = 224 * 1024 / BLOCKS - 1024 - mods;   // one block's rings
+    depth = budget >= 8 * 3 * row ? 3 : budget >= 8 * 2 * row ? 2 : 1;
+    const long long per_wave = 8LL * BLOCKS * sms;
+    rpw = (int)std::min((rows + per_wave - 1) / per_wave, 64LL);
+  }
+  const unsigned grid = (unsigned)((rows + 8LL * rpw - 1) / (8LL * rpw));
+  const size_t smem = (size_t)(mods + 8 * depth * row);
+  auto go = [&](auto kernel) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (a != cudaSuccess) return a;
+    }
+    launch_pdl(kernel, dim3(grid), dim3(256), smem, s, x, out, rows, C, shift, scale, mod_stride, seg_split, rpb0,
+               rpb1, rpw);
+    return launched();
+  };
+  return depth == 3 ? go(k_ln_mod<T, NCH, 3>) : depth == 2 ? go(k_ln_mod<T, NCH, 2>) : go(k_ln_mod<T, NCH, 1>);
 }
 
 template <class T>
 static cudaError_t ln_mod_t(const void* x, void* out, long long rows, int C, const float* shift, const float* scale,
                             int mod_stride, int seg_split, int rpb0, int rpb1, cudaStream_t s) {
-  constexpr int V = VecN<T>::n;
-  const int nch = (C / V + 31) / 32;
-  // rows per warp: one while a row per warp makes at most about two waves
-  // of blocks (every row's loads in flight at once), else enough that the
-  // blocks fill about two per SM (measured: 4096 x 1152 rows 6.6 us with one
-  // row per warp, 8.5 us with two; 14310 x 2048 rows 32.5 us with one, 24.5
-  // us with six)
-  const long long per_wave = 8LL * 2 * num_sms();
-  int rpw = rows <= 2 * per_wave ? 1 : (int)((rows + per_wave - 1) / per_wave);
-  rpw = rpw < 1 ? 1 : rpw > 8 ? 8 : rpw;
-  const unsigned grid = (unsigned)((rows + 8LL * rpw - 1) / (8LL * rpw));
-  const size_t smem = (size_t)2 * C * sizeof(float);  // shift + scale of one sample
-  if (C % 4 != 0 || smem > 48 * 1024) return cudaErrorInvalidValue;
+  const int nch = (C / VecN<T>::n + 31) / 32;
+  if (C % 4 != 0 || 2 * C * sizeof(float) > 48 * 1024) return cudaErrorInvalidValue;
   const T* xp = (const T*)x;
   T* op = (T*)out;
 #define FF_LN_CASE(n) \
-  case n:                                                                                                              \
-    if (rpw == 1)                                                                                                      \
-      launch_pdl(k_ln_mod1<T, n>, grid, 256, smem, s, xp, op, rows, C, shift, scale, mod_stride, seg_split, rpb0, rpb1); \
-    else                                                                                                               \
-      launch_pdl(k_ln_mod<T, n>, grid, 256, smem, s, xp, op, rows, C, shift, scale, mod_stride, seg_split, rpb0, rpb1,  \
-                 rpw);                                                                                                 \
-    break;
+  case n: return ln_mod_launch<T, n>(xp, op, rows, C, shift, scale, mod_stride, seg_split, rpb0, rpb1, s);
   const int nchr = nch <= 6 ? nch : nch <= 8 ? 8 : nch <= 12 ? 12 : nch <= 16 ? 16 : 0;
   switch (nchr) {
     FF_LN_CASE(1) FF_LN_CASE(2) FF_LN_CASE(3) FF_LN_CASE(4) FF_LN_CASE(5) FF_LN_CASE(6)
@@ -685,7 +793,6 @@ static cudaError_t ln_mod_t(const void* x, void* out, long long rows, int C, con
       return cudaErrorInvalidValue;
   }
 #undef FF_LN_CASE
-  return launched();
 }
 
 cudaError_t launch_ln_mod(DType dt, const void* x, void* out, long long rows, int C, const float* shift,

@@ -1,4 +1,4 @@
-"""The fp32 CUDA-core kernels at the edges of their tiles and dispatch rules,
+"""The fp32 CUDA-core kernels and the row-wise LayerNorm at the edges of their tiles and dispatch rules,
 against float64."""
 
 import pytest
@@ -73,3 +73,22 @@ def test_f32_attention(cuda, dtype, B, nt, ni, H, d, pad):
     ref = (torch.softmax(q @ k.transpose(2, 3) / d ** 0.5, -1) @ v).transpose(1, 2).reshape(B, n, C)
     assert rel_l2(f64(out)[rows], ref.numpy()) < (2e-6 if dtype == "f32" else 4e-3)
     assert torch.all(out[-1] == 3.0)
+
+
+# ring depths and blocks per SM of every width class, samples that change inside
+# a block, a last block and warp with few rows, one row; unused row kept
+LN = [("bf16", 1, 3072, 1), ("bf16", 4900, 128, 700), ("bf16", 6001, 1152, 250), ("bf16", 5003, 2048, 5003),
+      ("bf16", 5000, 3072, 33), ("bf16", 77, 4096, 20), ("f32", 4999, 1536, 1000), ("f32", 5001, 2048, 7)]
+
+
+@pytest.mark.parametrize("dtype,rows,C,rpb", LN)
+def test_ln_ring(cuda, dtype, rows, C, rpb):
+    x = randn((rows, C), dtype, 1, 2.0) + 3.0
+    mod = randn(((rows + rpb - 1) // rpb, 2 * C), "f32", 2, 0.1)
+    out = torch.full((rows + 1, C), 9.0, dtype=x.dtype, device=cuda)
+    ff.featfix_op_ln_modulate(dtype, x, out[:rows], rows, C, mod[:, :C], mod[:, C:], 2 * C, rpb)
+    torch.cuda.synchronize()
+    b = torch.arange(rows).numpy() // rpb
+    ref = oracle.model.layer_norm(f64(x)) * (1 + f64(mod)[b, C:]) + f64(mod)[b, :C]
+    assert rel_l2(f64(out)[:rows], ref) < (2e-6 if dtype == "f32" else 4e-3)
+    assert torch.all(out[rows] == 9.0)
