@@ -96,6 +96,10 @@ SIGNATURES = {
     "featfix_op_attention": (_I, [_I, _VP, _I, _VP, _I, _I, _I, _I, _I, _I, _VP]),
 }
 
+# argument arrays of the draft and the paid check (at most four history terms)
+_PTRS = [_VP * n for n in range(5)]
+_DOUBLES = [_D * n for n in range(5)]
+
 _lib = None
 
 
@@ -118,19 +122,37 @@ def _ptr(t):
     """Device (or host) address of a tensor / ndarray / int; None -> NULL."""
     if t is None:
         return None
-    if isinstance(t, int):
-        return t
     if hasattr(t, "data_ptr"):
         return t.data_ptr()
+    if isinstance(t, int):
+        return t
     if hasattr(t, "ctypes"):
         return t.ctypes.data
     raise TypeError("cannot take the address of %r" % type(t))
 
 
+_raw_stream = None
+
+
+def _current_stream():
+    """Handle of PyTorch's current stream.  The raw lookup where this PyTorch
+    has it: torch.cuda.current_stream() builds a Stream object on every call,
+    about 1.5 us of a 10 us op call."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        else:
+            device = torch.cuda.current_device
+            _raw_stream = lambda: raw(device())
+    return _raw_stream()
+
+
 def _stream_ptr(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -360,9 +382,16 @@ def _dt(dtype):
     return DTYPE[dtype] if isinstance(dtype, str) else int(dtype)
 
 
+def _hist_args(hist, w):
+    """(pointer array, weight array) of the history terms."""
+    n = len(hist)
+    if n < len(_PTRS):
+        return _PTRS[n](*[_ptr(h) for h in hist]), _DOUBLES[n](*map(float, w))
+    return (_VP * n)(*[_ptr(h) for h in hist]), (_D * n)(*map(float, w))
+
+
 def featfix_op_draft(dtype, x, hist, w, stream=None):
-    hp = (_VP * len(hist))(*[_ptr(h) for h in hist])
-    wa = (_D * len(hist))(*[float(v) for v in w])
+    hp, wa = _hist_args(hist, w)
     _check(lib().featfix_op_draft(_dt(dtype), _ptr(x), hp, wa, len(hist), x.numel(), _stream_ptr(stream)))
 
 
@@ -371,8 +400,7 @@ def featfix_op_verify_workspace(n):
 
 
 def featfix_op_verify(dtype, u, hist, w, hf, sums, workspace, write_draft=False, stream=None):
-    hp = (_VP * len(hist))(*[_ptr(h) for h in hist])
-    wa = (_D * len(hist))(*[float(v) for v in w])
+    hp, wa = _hist_args(hist, w)
     _check(lib().featfix_op_verify(_dt(dtype), _ptr(u), hp, wa, len(hist), _ptr(hf), u.numel(), int(write_draft),
                                    _ptr(sums), _ptr(workspace), workspace.numel() * workspace.element_size(),
                                    _stream_ptr(stream)))
@@ -381,8 +409,7 @@ def featfix_op_verify(dtype, u, hist, w, hf, sums, workspace, write_draft=False,
 def featfix_op_verify_noalloc(dtype, u, hist, w, hf, sums, write_draft=False, stream=None):
     """featfix_op_verify with the library's fixed scratch array (no device
     allocation by anyone); see include/featfix_ops.h."""
-    hp = (_VP * len(hist))(*[_ptr(h) for h in hist])
-    wa = (_D * len(hist))(*[float(v) for v in w])
+    hp, wa = _hist_args(hist, w)
     _check(lib().featfix_op_verify_noalloc(_dt(dtype), _ptr(u), hp, wa, len(hist), _ptr(hf), u.numel(),
                                            int(write_draft), _ptr(sums), _stream_ptr(stream)))
 
