@@ -764,16 +764,22 @@ static cudaError_t ln_mod_launch(const T* x, T* out, long long rows, int C, cons
   }
   const unsigned grid = (unsigned)((rows + 8LL * rpw - 1) / (8LL * rpw));
   const size_t smem = (size_t)(mods + 8 * depth * row);
-  auto go = [&](auto kernel) -> cudaError_t {
-    if (smem > 48 * 1024) {
-      const cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (a != cudaSuccess) return a;
-    }
+  // The kernel attribute belongs to the process, so it is the instance's own
+  // largest size, whatever this call needs: threads with rows of other widths
+  // set the same value.
+  auto go = [&](auto kernel, auto d) -> cudaError_t {
+    constexpr int ROW_MAX = NCH * 32 * 16, MODS_MAX = NCH * 32 * VecN<T>::n * 8;
+    constexpr int SMEM_MAX = MODS_MAX + 8 * decltype(d)::value * ROW_MAX;
+    static_assert(SMEM_MAX <= 227 * 1024, "shared memory of a block");
+    const cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    if (a != cudaSuccess) return a;
     launch_pdl(kernel, dim3(grid), dim3(256), smem, s, x, out, rows, C, shift, scale, mod_stride, seg_split, rpb0,
                rpb1, rpw);
     return launched();
   };
-  return depth == 3 ? go(k_ln_mod<T, NCH, 3>) : depth == 2 ? go(k_ln_mod<T, NCH, 2>) : go(k_ln_mod<T, NCH, 1>);
+  return depth == 3   ? go(k_ln_mod<T, NCH, 3>, std::integral_constant<int, 3>())
+         : depth == 2 ? go(k_ln_mod<T, NCH, 2>, std::integral_constant<int, 2>())
+                      : go(k_ln_mod<T, NCH, 1>, std::integral_constant<int, 1>());
 }
 
 template <class T>

@@ -1,6 +1,8 @@
 """The fp32 CUDA-core kernels and the row-wise LayerNorm at the edges of their tiles and dispatch rules,
 against float64."""
 
+import threading
+
 import pytest
 import torch
 
@@ -92,3 +94,33 @@ def test_ln_ring(cuda, dtype, rows, C, rpb):
     ref = oracle.model.layer_norm(f64(x)) * (1 + f64(mod)[b, C:]) + f64(mod)[b, :C]
     assert rel_l2(f64(out)[:rows], ref) < (2e-6 if dtype == "f32" else 4e-3)
     assert torch.all(out[rows] == 9.0)
+
+
+# Two threads, each with its own stream and row width, on one kernel instance:
+# no call's launch may depend on the other's.  (The calls go through the C entry
+# point with prepared arguments, so that they overlap.)
+def test_ln_threads(cuda):
+    rows, outs, calls, failed = 5000, [], [], [0, 0]
+    for i, C in enumerate((1288, 1384)):
+        x, mod = randn((rows, C), "bf16", 1, 2.0), randn((1, 2 * C), "f32", 2, 0.1)
+        out, stream = torch.zeros_like(x), torch.cuda.Stream()
+        ref = oracle.model.layer_norm(f64(x)) * (1 + f64(mod)[0, C:]) + f64(mod)[0, :C]
+        outs.append((out, ref, x, mod, stream))
+        calls.append((ff.DTYPE["bf16"], x.data_ptr(), out.data_ptr(), rows, C, mod.data_ptr(), mod.data_ptr() + 4 * C,
+                      2 * C, rows, stream.cuda_stream))
+    torch.cuda.synchronize()
+
+    def work(i):
+        op = ff.lib().featfix_op_ln_modulate
+        for _ in range(6000):
+            failed[i] += op(*calls[i]) != 0
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert failed == [0, 0]
+    for out, ref, *_ in outs:
+        assert rel_l2(f64(out), ref) < 4e-3
