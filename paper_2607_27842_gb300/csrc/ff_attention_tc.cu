@@ -56,10 +56,15 @@ using namespace tc;
 constexpr int AQ = 128;        // queries per tile (MMA M)
 constexpr int AKV = 128;       // keys per tile (MMA N of S, K of P V)
 constexpr float RESCALE_LOG2 = 8.0f;
-// a half tile's sum of speculative exponentials that still stands: P, O and the
-// row sum keep their relative precision at any scale, and N such tiles times
-// any bf16-sized value stay far from overflow
-constexpr float SPEC_LIMIT = 1073741824.0f;   // 2^30
+// A half tile's sum of speculative exponentials that still stands: 2^RESCALE_LOG2
+// for each of its keys, which is also as far as a reference taken from the
+// tile's max lets P grow.  So O before the division stays below keys (whole
+// tiles) * 2^8 * |v|, and is finite for |v| up to about 2^120 / keys.  (With 2^30,
+// values of 2^104 overflowed where scores grow along 4096 keys; with 2^8, half tiles
+// are made again more often: 14566 tokens with normal scores of standard
+// deviation 3 1205 -> 1429 us.)
+constexpr float SPEC_LIMIT = 16384.0f;
+static_assert(SPEC_LIMIT == AKV / 2 * 256 && RESCALE_LOG2 == 8.0f, "2^RESCALE_LOG2 for each key of a half tile");
 constexpr int SHORT_KV_TILES = 4;  // sequences of at most 4 x 128 tokens: one query tile per CTA
 constexpr size_t SMEM_LIMIT = 232448;  // opt-in dynamic shared memory per block
 
