@@ -155,8 +155,9 @@ struct EpiWarp {
 // registers or branches for the others:
 //   EPI_FULL    gate, residual, history increment (any of them);
 //   EPI_PLAIN   bias, RoPE, activation only (qkv, fc1, linear1);
-//   EPI_SINGLE  EPI_FULL with a residual where every CTA holds one tile, so
-//               nothing hides the epilogue (epi_single below).
+//   EPI_SINGLE  EPI_FULL with a residual or a history increment where every
+//               CTA holds one tile, so nothing hides the epilogue (epi_single
+//               below).
 enum { EPI_FULL = 0, EPI_PLAIN = 1, EPI_SINGLE = 2 };
 
 // The epilogue of one tile, inlined once per problem of the launch so that
@@ -586,15 +587,15 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
   uint8_t* const ep = W.ep;
   uint8_t* const ring = W.smem + (W.warp - 2) * 16384;    // 12 KB of blocks, 1.5 KB of constants
   uint64_t* const rbar = &W.rbar[W.warp - 2];
-  const bool hist = e.hist_out != nullptr;
+  const bool hist = e.hist_out != nullptr, res = e.resid != nullptr;   // one of them at least
   // block i: output rows y0 .. y0 + 31, columns x0 .. x0 + 31
   const int xb = t.sw ? t.n0 + q * 32 : t.n0 + W.c_lo, yb = t.sw ? t.m0 + h * (BN / 2) : t.m0 + q * 32;
   const int dx = t.sw ? 0 : 32, dy = t.sw ? 32 : 0;
   const int nb = xb < N && yb < M ? min(4, t.sw ? (M - yb + 31) >> 5 : (N - xb + 31) >> 5) : 0;
   auto rblk = [&](int i) { return i < 2 ? ep + i * 2048 : ring + (i - 2) * 2048; };
   auto hblk = [&](int i) { return ring + 4096 + i * 2048; };
-  const int early = min(nb, 2);
-  if (lane == 0 && nb > 0) {
+  const int early = res ? min(nb, 2) : 0;
+  if (lane == 0 && early > 0) {
     mbar_expect_tx(rbar, early * 2048u);
     for (int i = 0; i < early; ++i) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
   }
@@ -614,7 +615,7 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
   int ok = 1;
   if (lane == 0) {
     ok = mbar_wait_p(W.tfull, 0, W.abort_flag) ? 1 : 0;
-    if (nb > 0) {  // the early blocks (they land before the CTA exits, also after a failed wait)
+    if (early > 0) {  // the early blocks (they land before the CTA exits, also after a failed wait)
       const unsigned long long t0 = gtimer();
       while (!mbar_try(rbar, 0))
         if (gtimer() - t0 > WAIT_LIMIT_NS) { atomicOr(&g_watchdog, 2u); *W.abort_flag = 1; ok = 0; break; }
@@ -623,20 +624,28 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
   ok = __shfl_sync(0xffffffffu, ok, 0);
   if (!ok) return false;
   tc_fence_after();
-  const bool late = nb > 2 || (hist && nb > 0);
-  if (lane == 0 && late) {
-    mbar_expect_tx(rbar, (uint32_t)((nb - early) + (hist ? nb : 0)) * 2048u);
+  const int late = (res ? nb - early : 0) + (hist ? nb : 0);
+  if (lane == 0 && late > 0) {
+    mbar_expect_tx(rbar, late * 2048u);
     for (int i = 0; i < nb; ++i) {
       if (hist) tma_load(tmHB, rbar, hblk(i), xb + i * dx, yb + i * dy);
-      if (i >= 2) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
+      if (res && i >= 2) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
     }
   }
-  bool late_wait = late;
+  if (!res) {  // a residual of -0, which adds nothing, so the loops below need no second form (a branch there: 2%)
+    for (int i = 0; i < nb; ++i)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<uint4*>(rblk(i) + blk_off(lane, k)) =
+            make_uint4(0x80008000u, 0x80008000u, 0x80008000u, 0x80008000u);
+    __syncwarp();
+  }
+  bool late_wait = late > 0;
   auto late_ready = [&]() -> bool {
     if (!late_wait) return true;
     late_wait = false;
     int w = 1;
-    if (lane == 0) w = mbar_wait_p(rbar, 1, W.abort_flag) ? 1 : 0;
+    if (lane == 0) w = mbar_wait_p(rbar, early > 0 ? 1 : 0, W.abort_flag) ? 1 : 0;
     return __shfl_sync(0xffffffffu, w, 0) != 0;
   };
   const uint32_t tq = W.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * (BN / 2));
@@ -1323,7 +1332,8 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
     if (tm.staged && t256 <= g_sms) {
       if (e.resid && make_store_map(&mr, const_cast<void*>(e.resid), M, N, e.ld_resid)) tm.pre |= 1;
       if (e.hist_out && make_store_map(&mhb, const_cast<void*>(e.hist_base), M, N, e.ldo)) tm.pre |= 2;
-      if ((tm.pre & 1) && (!e.hist_out || (tm.pre & 2)) && !e.rope && e.act != 2 && e.act_col0 == 0) epi = EPI_SINGLE;
+      const bool blocks = (!e.resid || (tm.pre & 1)) && (!e.hist_out || (tm.pre & 2)) && tm.pre;
+      if (blocks && !e.rope && e.act != 2 && e.act_col0 == 0) epi = EPI_SINGLE;
     }
     const int grid = (int)(t256 < g_sms ? t256 : g_sms);
     const TileMap none = {};

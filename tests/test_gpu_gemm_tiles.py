@@ -82,3 +82,22 @@ def test_gemm_single_tile(cuda, M, N, K, rpb, epilogue, shift):
     assert torch.all(buf[M] == 5.0) and torch.all(hist[M] == 5.0)
     if epilogue == "gated_history":
         assert rel_l2(f64(hist)[:M], f64(out) - f64(base)) < 4e-3
+
+
+# one tile per CTA with a history increment and no residual (nothing to load
+# before the accumulator is ready): as above
+@pytest.mark.parametrize("M,N,K,rpb", [(2300, 1800, 136, 500), (250, 520, 72, 33), (130, 392, 1152, 130), (40, 48, 64, 32)])
+@pytest.mark.parametrize("gated", [False, True])
+def test_gemm_single_tile_history_only(cuda, M, N, K, rpb, gated):
+    a, w, bias, base = randn((M, K), "bf16", 1), randn((N, K), "bf16", 2, 0.1), randn(N, "bf16", 3), randn((M, N), "bf16", 9)
+    buf = torch.full((2, M + 1, N), 5.0, dtype=torch.bfloat16, device=cuda)
+    y, kw = f64(a) @ f64(w).T + f64(bias), {}
+    if gated:
+        gate = randn((-(-M // rpb), N), "f32", 7)
+        kw = dict(gate=gate, gate_stride=N, rows_per_batch=rpb)
+        y = y * f64(gate)[torch.arange(M).numpy() // rpb]
+    ff.featfix_op_gemm("bf16", a, w, buf[0, :M], bias=bias, hist_base=base, hist_out=buf[1, :M], **kw)
+    torch.cuda.synchronize()
+    assert rel_l2(f64(buf[0, :M]), y) < 4e-3
+    assert rel_l2(f64(buf[1, :M]), f64(buf[0, :M]) - f64(base)) < 4e-3
+    assert torch.all(buf[:, M] == 5.0)
