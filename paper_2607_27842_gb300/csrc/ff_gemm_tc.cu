@@ -1257,18 +1257,22 @@ bool staged_maps(const EpiArgs& e, int M, int N, CUtensorMap* mo, CUtensorMap* m
 // MMA; 14310 x 6144 x 2048 219 -> 199 us, 4608 x 3072 x 2048 51 -> 43, 4096 x
 // 4608 x 1152 with GELU 33.8 -> 29.5), so pairs run wherever they need no more
 // waves; within one wave short reductions stay with single CTAs, whose
-// epilogue blocks come by TMA (1024 x 4608 x 256 9.2 against 9.5 us).
+// epilogue blocks come by TMA (1024 x 4608 x 256 9.2 against 9.5 us), up to a K
+// of 1024 and with a history increment, whose epilogue is the longest, of 4096
+// (singles against pairs, gate, residual and history: 1103 x 3624 x 2296 29.7
+// and 38.1 us, 1485 x 1816 x 3864 7% apart; without history, 718 x 5768 x 4744,
+// pairs take 14% less).
 // 128-wide pair tiles take 0.85 of a 256-wide tile's time, so they pay only
 // where the 256-wide tiles leave half the pairs idle; counted at half the time
 // they took 8192 x 8192 x 8192, 945 us against 590.
-int pair_bn(long long m256, long long t128x256, int N, int K, int sms) {
+int pair_bn(long long m256, long long t128x256, int N, int K, bool hist, int sms) {
   const int pairs = sms / 2;
   const long long w_single = (t128x256 + sms - 1) / sms;
   const long long w256 = (m256 * ((N + 255) / 256) + pairs - 1) / pairs;
   const long long w128 = (m256 * ((N + 127) / 128) + pairs - 1) / pairs;
   if (w256 > w_single) return 0;
   if (w128 <= w256) return 128;
-  return w256 > 1 || K >= 1024 ? 256 : 0;
+  return w256 > 1 || K >= (hist ? 4096 : 1024) ? 256 : 0;
 }
 
 // The single-CTA kernel's 128 x 256 tiles, remainder columns in swapped tiles.
@@ -1287,7 +1291,7 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
   if (!ln_ok(e, N)) return cudaErrorInvalidValue;
   if (((uintptr_t)A & 15) || ((uintptr_t)W & 15)) return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
-  const int bn = M >= 2 * BM ? pair_bn((M + 2 * BM - 1) / (2 * BM), wide_tiles(M, N), N, K, g_sms) : 0;
+  const int bn = M >= 2 * BM ? pair_bn((M + 2 * BM - 1) / (2 * BM), wide_tiles(M, N), N, K, e.hist_out != nullptr, g_sms) : 0;
   if (bn) {
     const int pairs = g_sms / 2;
     if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, bn / 2)) return cudaErrorInvalidValue;
@@ -1381,7 +1385,7 @@ cudaError_t gemm_tc_grouped(int M0, const void* A0, const void* W0, const EpiArg
   // both problems in one CTA-pair launch (256-row tiles of the text rows,
   // then of the image rows)
   const long long rows_t = ((M0 + 2 * BM - 1) / (2 * BM)) + ((M1 + 2 * BM - 1) / (2 * BM));
-  const int bn = M0 >= 2 * BM ? pair_bn(rows_t, wide_tiles(M0, N) + wide_tiles(M1, N), N, K, g_sms) : 0;
+  const int bn = M0 >= 2 * BM ? pair_bn(rows_t, wide_tiles(M0, N) + wide_tiles(M1, N), N, K, false, g_sms) : 0;
   if (bn) {
     if (K % 8 != 0 || lda % 8 != 0 || ldw % 8 != 0 || N % 8 != 0) return cudaErrorInvalidValue;
     if (((uintptr_t)A0 & 15) || ((uintptr_t)W0 & 15) || ((uintptr_t)A1 & 15) || ((uintptr_t)W1 & 15))

@@ -11,22 +11,45 @@ from paper_2607_27842_gb300 import featfix as ff
 from .gpu_helpers import rel_l2
 from .test_gpu_ops import f64, randn
 
-pytestmark = pytest.mark.gpu
+# The kernel a layer takes, restated from the dispatch: "pair128", "pair256" (CTA
+# pairs, tiles 128 or 256 columns wide), "single" (a tile per CTA: its own
+# epilogue where there is a residual or a history increment), "singles" (several
+# tiles per CTA).  Outputs and gates of these tests allow the staged epilogues
+# (16-byte aligned rows, at least 32 rows per gate sample).
+def kernel(M, N, K, hist, sms):
+    def waves(tiles, slots):
+        return -(-tiles // slots)
+    rem, m256 = N % 256, -(-M // 256)
+    wide = -(-M // 128) * (N // 256) + (-(-rem // 128) * m256 if rem else 0)
+    w256, w128 = (waves(m256 * -(-N // bn), sms // 2) for bn in (256, 128))
+    if M >= 256 and w256 <= waves(wide, sms):
+        if w128 <= w256:
+            return "pair128"
+        if w256 > 1 or K >= (4096 if hist else 1024):
+            return "pair256"
+    return "single" if wide <= sms else "singles"
 
-# M, N, K, rows per gate sample
-SHAPES = [(256, 32, 64, 256),        # pairs, one 128-wide tile, mostly empty
-          (257, 136, 72, 40),        # a second row block of one row, 8 remainder columns
-          (255, 256, 64, 255),       # one row short of a pair: single CTAs
-          (511, 264, 8, 32),         # one k-step of 8
-          (1024, 4608, 256, 256),    # one wave, short reduction: single CTAs
-          (1024, 4608, 1024, 200),   # one wave, pairs
-          (2300, 1800, 136, 500),    # nine row blocks: two groups, the last of one block
-          (4352, 3464, 72, 4352)]    # 17 row blocks, three waves
+
+# M, N, K, rows per gate sample, kernel without and with a history increment
+SHAPES = [(256, 32, 64, 256, "pair128", "pair128"),        # one tile, mostly empty
+          (257, 136, 72, 40, "pair128", "pair128"),        # a second row block of one row, 8 remainder columns
+          (255, 256, 64, 255, "single", "single"),         # one row short of a pair
+          (511, 264, 8, 32, "pair128", "pair128"),         # one k-step of 8
+          (1024, 4608, 256, 256, "single", "single"),      # one wave, short reduction
+          (1024, 4608, 1024, 200, "pair256", "single"),    # one wave, longer reduction
+          (512, 8200, 4096, 200, "pair256", "pair256"),    # one wave, 8 remainder columns, K of 4096
+          (2300, 1800, 136, 500, "single", "single"),      # remainder columns in swapped tiles
+          (1000, 1160, 64, 100, "pair128", "pair128"),     # warps and blocks whose rows lie in two samples
+          (300, 1288, 72, 33, "pair128", "pair128"),
+          (900, 904, 136, 900, "pair128", "pair128"),
+          (4333, 2056, 72, 100, "singles", "singles"),     # two waves where pairs would need three
+          (4352, 3464, 72, 4352, "pair256", "pair256")]    # 17 row blocks: two full groups of eight and one
 
 
 # the result is stored in bf16 (2^-9 relative, 1.7e-3 in the norm), the
 # increment is the difference of two stored values rounded again
-@pytest.mark.parametrize("M,N,K,rpb", SHAPES)
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,rpb", [c[:4] for c in SHAPES])
 @pytest.mark.parametrize("epilogue", ["bias", "gelu", "gated", "gated_history"])
 def test_gemm_tiles(cuda, M, N, K, rpb, epilogue):
     a, w, bias = randn((M, K), "bf16", 1), randn((N, K), "bf16", 2, 0.1), randn(N, "bf16", 3)
@@ -53,11 +76,27 @@ def test_gemm_tiles(cuda, M, N, K, rpb, epilogue):
         assert torch.all(hist[M] == 5.0)
 
 
-# one tile per CTA with a residual: normal and swapped tiles, blocks cut by M
-# and N, warps and blocks whose rows lie in two samples, bias and gate that are
-# not 16-byte aligned
-@pytest.mark.parametrize("M,N,K,rpb", [(4096, 1152, 200, 256), (1000, 1160, 64, 100), (300, 1288, 72, 33),
-                                       (130, 392, 1152, 130), (900, 904, 136, 900), (96, 264, 64, 32)])
+# one tile per CTA: normal and swapped tiles, blocks cut by M and N, warps and
+# blocks whose rows lie in two samples (rows per sample not multiples of 32)
+SINGLE = [(4096, 1152, 200, 256), (130, 392, 1152, 130), (96, 264, 64, 32), (250, 520, 72, 33), (200, 1288, 64, 50),
+          (255, 136, 64, 45), (2300, 1800, 136, 500)]
+# the same forms on CTA pairs
+PAIRED = [(1000, 1160, 64, 100), (300, 1288, 72, 33), (900, 904, 136, 900)]
+
+
+@pytest.mark.parametrize("sms", [148, 152])
+def test_cases_select_their_kernel(sms):
+    for M, N, K, _, plain, hist in SHAPES:
+        assert (kernel(M, N, K, False, sms), kernel(M, N, K, True, sms)) == (plain, hist), (M, N, K)
+    for M, N, K, _ in SINGLE:
+        assert kernel(M, N, K, False, sms) == kernel(M, N, K, True, sms) == "single", (M, N, K)
+    for M, N, K, _ in PAIRED:
+        assert kernel(M, N, K, False, sms) == kernel(M, N, K, True, sms) == "pair128", (M, N, K)
+
+
+# bias and gate 16-byte aligned or not
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,rpb", SINGLE + PAIRED)
 @pytest.mark.parametrize("epilogue", ["resid", "gelu_gated", "gated_history"])
 @pytest.mark.parametrize("shift", [0, 1])
 def test_gemm_single_tile(cuda, M, N, K, rpb, epilogue, shift):
@@ -86,6 +125,7 @@ def test_gemm_single_tile(cuda, M, N, K, rpb, epilogue, shift):
 
 # one tile per CTA with a history increment and no residual (nothing to load
 # before the accumulator is ready): as above
+@pytest.mark.gpu
 @pytest.mark.parametrize("M,N,K,rpb", [(2300, 1800, 136, 500), (250, 520, 72, 33), (130, 392, 1152, 130), (40, 48, 64, 32)])
 @pytest.mark.parametrize("gated", [False, True])
 def test_gemm_single_tile_history_only(cuda, M, N, K, rpb, gated):
