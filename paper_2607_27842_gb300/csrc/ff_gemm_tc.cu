@@ -155,10 +155,10 @@ struct EpiWarp {
 // registers or branches for the others:
 //   EPI_FULL    gate, residual, history increment (any of them);
 //   EPI_PLAIN   bias, RoPE, activation only (qkv, fc1, linear1);
-//   EPI_SINGLE  EPI_FULL with a residual or a history increment where every
-//               CTA holds one tile, so nothing hides the epilogue (epi_single
-//               below).
-enum { EPI_FULL = 0, EPI_PLAIN = 1, EPI_SINGLE = 2 };
+//   EPI_SINGLE  EPI_FULL with a residual where every CTA holds one tile, so
+//               nothing hides the epilogue (epi_single below);
+//   EPI_SINGLE_HIST  the same with a history increment and no residual.
+enum { EPI_FULL = 0, EPI_PLAIN = 1, EPI_SINGLE = 2, EPI_SINGLE_HIST = 3 };
 
 // The epilogue of one tile, inlined once per problem of the launch so that
 // every EpiArgs / TileMap field and tensor map is read from its own kernel
@@ -579,7 +579,7 @@ __device__ __forceinline__ int sample_end(const EpiArgs& e, int r) {
 // Against the shared form with its block-by-block buffers, shuffled bias and
 // gate and transposed swapped tiles: 4096 x 1152 x 1152 (gate, residual) 19.3
 // -> 14.5 us, 4096 x 1152 x 4608 (and history) 46.2 -> 41.0 us.
-template <int BN>
+template <int BN, bool RES>
 __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, const int M, const int N, const TileAt t,
                                            const CUtensorMap* tmO, const CUtensorMap* tmH, const CUtensorMap* tmR,
                                            const CUtensorMap* tmHB) {
@@ -587,14 +587,14 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
   uint8_t* const ep = W.ep;
   uint8_t* const ring = W.smem + (W.warp - 2) * 16384;    // 12 KB of blocks, 1.5 KB of constants
   uint64_t* const rbar = &W.rbar[W.warp - 2];
-  const bool hist = e.hist_out != nullptr, res = e.resid != nullptr;   // one of them at least
+  const bool hist = !RES || e.hist_out != nullptr;
   // block i: output rows y0 .. y0 + 31, columns x0 .. x0 + 31
   const int xb = t.sw ? t.n0 + q * 32 : t.n0 + W.c_lo, yb = t.sw ? t.m0 + h * (BN / 2) : t.m0 + q * 32;
   const int dx = t.sw ? 0 : 32, dy = t.sw ? 32 : 0;
   const int nb = xb < N && yb < M ? min(4, t.sw ? (M - yb + 31) >> 5 : (N - xb + 31) >> 5) : 0;
   auto rblk = [&](int i) { return i < 2 ? ep + i * 2048 : ring + (i - 2) * 2048; };
   auto hblk = [&](int i) { return ring + 4096 + i * 2048; };
-  const int early = res ? min(nb, 2) : 0;
+  const int early = RES ? min(nb, 2) : 0;
   if (lane == 0 && early > 0) {
     mbar_expect_tx(rbar, early * 2048u);
     for (int i = 0; i < early; ++i) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
@@ -624,28 +624,20 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
   ok = __shfl_sync(0xffffffffu, ok, 0);
   if (!ok) return false;
   tc_fence_after();
-  const int late = (res ? nb - early : 0) + (hist ? nb : 0);
+  const int late = (RES ? nb - early : 0) + (hist ? nb : 0);
   if (lane == 0 && late > 0) {
     mbar_expect_tx(rbar, late * 2048u);
     for (int i = 0; i < nb; ++i) {
       if (hist) tma_load(tmHB, rbar, hblk(i), xb + i * dx, yb + i * dy);
-      if (res && i >= 2) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
+      if (RES && i >= 2) tma_load(tmR, rbar, rblk(i), xb + i * dx, yb + i * dy);
     }
-  }
-  if (!res) {  // a residual of -0, which adds nothing, so the loops below need no second form (a branch there: 2%)
-    for (int i = 0; i < nb; ++i)
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        *reinterpret_cast<uint4*>(rblk(i) + blk_off(lane, k)) =
-            make_uint4(0x80008000u, 0x80008000u, 0x80008000u, 0x80008000u);
-    __syncwarp();
   }
   bool late_wait = late > 0;
   auto late_ready = [&]() -> bool {
     if (!late_wait) return true;
     late_wait = false;
     int w = 1;
-    if (lane == 0) w = mbar_wait_p(rbar, early > 0 ? 1 : 0, W.abort_flag) ? 1 : 0;
+    if (lane == 0) w = mbar_wait_p(rbar, RES ? 1 : 0, W.abort_flag) ? 1 : 0;
     return __shfl_sync(0xffffffffu, w, 0) != 0;
   };
   const uint32_t tq = W.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * (BN / 2));
@@ -692,12 +684,12 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         uint4* const rp = reinterpret_cast<uint4*>(rblk(i) + blk_off(lane, k));
-        const uint4 r4 = *rp;
+        const uint4 r4 = RES ? *rp : make_uint4(0, 0, 0, 0);
         const uint32_t rr[4] = {r4.x, r4.y, r4.z, r4.w};
         uint32_t ob[4];
 #pragma unroll
         for (int z = 0; z < 4; ++z) {
-          const unsigned long long a = fadd2(y[4 * k + z], bf2u(rr[z]));
+          const unsigned long long a = RES ? fadd2(y[4 * k + z], bf2u(rr[z])) : y[4 * k + z];
           ob[z] = pack2(lo_f(a), hi_f(a));
         }
         *rp = make_uint4(ob[0], ob[1], ob[2], ob[3]);
@@ -740,8 +732,10 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
       // behind the write before it (37 x 48 x 1192, residual and history 13.6 -> 11.1 us,
       // 4096 x 1152 x 4608 with gate, residual and history 43.0 -> 41.0)
       auto at = [&](uint8_t* blk, int j) { return reinterpret_cast<bf16*>(blk + j * 64 + off[(j >> 1) & 3]); };
+      if constexpr (RES) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] += __bfloat162float(*at(rblk(i), j));
+        for (int j = 0; j < 32; ++j) v[j] += __bfloat162float(*at(rblk(i), j));
+      }
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const bf16 o = __float2bfloat16_rn(v[j]);
@@ -913,8 +907,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1;
       bool ok;
-      if constexpr (EPI == EPI_SINGLE) {
-        ok = epi_single<BN>(W, e0, M0, N, tile_at<BN>(tm0, tile), &tmO, &tmH, &tmR, &tmHB);
+      if constexpr (EPI == EPI_SINGLE || EPI == EPI_SINGLE_HIST) {
+        ok = epi_single<BN, EPI == EPI_SINGLE>(W, e0, M0, N, tile_at<BN>(tm0, tile), &tmO, &tmH, &tmR, &tmHB);
       } else if constexpr (GROUPED) {
         ok = tile < n1 ? epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN, EPI>(W, e1, tm1, M1, N, tile_at<BN>(tm1, tile), acc, aph, epi_cnt, &tmO1,
                                             &tmH1, &tmR, &tmHB)
@@ -1150,8 +1144,10 @@ auto gemm_fn(int ln, int epi) -> decltype(&k_gemm_tc<BN, G, 0, EPI_FULL>) {
   if (ln == 2) return k_gemm_tc<BN, G, 2, EPI_FULL>;
   if constexpr (BN == 256) {
     if (epi == EPI_PLAIN) return k_gemm_tc<BN, G, 0, EPI_PLAIN>;
-    if constexpr (!G)
+    if constexpr (!G) {
       if (epi == EPI_SINGLE) return k_gemm_tc<BN, G, 0, EPI_SINGLE>;
+      if (epi == EPI_SINGLE_HIST) return k_gemm_tc<BN, G, 0, EPI_SINGLE_HIST>;
+    }
   }
   return k_gemm_tc<BN, G, 0, EPI_FULL>;
 }
@@ -1197,7 +1193,7 @@ bool init_driver() {
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
     for (int ln = 0; ln < 3; ++ln)
-      for (int epi : {EPI_FULL, EPI_PLAIN, EPI_SINGLE}) {
+      for (int epi : {EPI_FULL, EPI_PLAIN, EPI_SINGLE, EPI_SINGLE_HIST}) {
         smem((const void*)gemm_fn<128, false>(ln, epi), Cfg<128>::SMEM);
         smem((const void*)gemm_fn<256, false>(ln, epi), Cfg<256>::SMEM);
         smem((const void*)gemm_fn<256, true>(ln, epi), Cfg<256>::SMEM);
@@ -1337,7 +1333,7 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
       if (e.resid && make_store_map(&mr, const_cast<void*>(e.resid), M, N, e.ld_resid)) tm.pre |= 1;
       if (e.hist_out && make_store_map(&mhb, const_cast<void*>(e.hist_base), M, N, e.ldo)) tm.pre |= 2;
       const bool blocks = (!e.resid || (tm.pre & 1)) && (!e.hist_out || (tm.pre & 2)) && tm.pre;
-      if (blocks && !e.rope && e.act != 2 && e.act_col0 == 0) epi = EPI_SINGLE;
+      if (blocks && !e.rope && e.act != 2 && e.act_col0 == 0) epi = e.resid ? EPI_SINGLE : EPI_SINGLE_HIST;
     }
     const int grid = (int)(t256 < g_sms ? t256 : g_sms);
     const TileMap none = {};
