@@ -473,8 +473,8 @@ cudaError_t launch_ln_ab(DType dt, const float* mod, long long mod_stride, int r
 // One warp per row, exact two-pass mean / variance from registers, one global
 // read and one write.
 // ---------------------------------------------------------------------------
-// One warp per row (8 rows per block, for row counts that fill about two
-// waves at most); the block first stages the shift /
+// One warp per row (8 rows per block, for row counts of one wave of resident
+// blocks); the block first stages the shift /
 // scale vectors of its first row's sample in shared memory (coalesced, read
 // back by every warp of that sample instead of 4 x 16 B per lane per chunk
 // from global memory).  Rows of up to six vectors per lane are held to 64
@@ -552,17 +552,20 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : 1) k_ln_mod1(const T* __re
   }
 }
 
-// Large row counts and wide rows: a block takes 8 * rpw consecutive rows, a warp
-// rpw of them in turn.  Rows reach the warp through its own ring of DEPTH slots in
+// Large row counts and wide rows: each block takes a share of the rows, its warps
+// every eighth of them.  Rows reach the warp through its own ring of DEPTH slots in
 // shared memory by cp.async (each lane copies and reads back its own vectors,
 // so a row needs no barrier), so DEPTH rows per warp are in flight while one is
 // reduced; the shift / scale of the block's first sample (read back by every
 // warp of that sample) are copied the same way behind the first rows, so the
-// two latencies overlap.  Bound by latency and bytes in flight, not by
-// arithmetic (packed fp32 pairs changed nothing at 14310 x 2048).  Against rows
-// held a register row ahead: 8704 x 3072 38.6 -> 25.7 us, 4608 x 3072 24.4 ->
-// 18.8, 8192 x 1152 16.9 -> 12.7, 14000 x 128 10.3 -> 4.9, 14310 x 2048 24.4 ->
-// 24.1.
+// two latencies overlap.  Written in packed fp32 pairs; scalar arithmetic was as
+// fast (14310 x 2048).
+// The blocks' shares differ by one row at most: in blocks of equal whole rows of
+// warps the last SMs run a block less or none (8000 x 2048: 334 blocks for 456
+// slots).  us with rows held a register row ahead, in equal blocks, as here: 8704 x
+// 3072 38.4, 25.8, 24.3; 4608 x 3072 22.2, 18.7, 15.1; 8000 x 2048 17.9, 19.1, 16.7;
+// 8192 x 1152 15.2, 10.3, 9.3; 14000 x 128 9.5, 5.1, 5.1; 14310 x 2048 24.9, 24.5,
+// 24.2 (4.8 TB/s).
 __device__ __forceinline__ void cp16_async(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
@@ -620,21 +623,23 @@ __device__ __forceinline__ uint4 packv(const f32x2 (&o)[4]) {
 template <class T, int NCH, int DEPTH>
 __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
     k_ln_mod(const T* __restrict__ x, T* __restrict__ out, long long rows, int C, const float* __restrict__ shift,
-             const float* __restrict__ scale, int mod_stride, int seg_split, int rpb0, int rpb1, int rpw) {
+             const float* __restrict__ scale, int mod_stride, int seg_split, int rpb0, int rpb1, int per, int rem) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ float4 smod4[];                  // [2 * C / 4]: shift, then scale; then the rings
   float* smod = reinterpret_cast<float*>(smod4);
   constexpr int V = VecN<T>::n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long r0 = (long long)blockIdx.x * 8 * rpw;
+  // the block's rows [r0, r0 + nb): per, one more in the first rem blocks
+  const long long r0 = (long long)blockIdx.x * per + min((int)blockIdx.x, rem);
+  const int nb = (int)min((long long)per + ((int)blockIdx.x < rem ? 1 : 0), rows - r0);
   const int b0 = (int)(r0 < seg_split ? r0 / rpb0 : (r0 - seg_split) / rpb1);
   const int nv = C / V;
-  const long long rw = r0 + (long long)warp * rpw;
-  const int n = (int)min((long long)rpw, rows - rw);  // the warp's rows (may be <= 0)
+  const long long rw = r0 + warp;                     // the warp's rows rw + 8 t, t < n (n may be 0)
+  const int n = (nb - warp + 7) >> 3;
   uint4* const ring = reinterpret_cast<uint4*>(smod4 + C / 2) + (size_t)warp * DEPTH * nv;
   auto copy_row = [&](int t) {
-    const uint4* xr = reinterpret_cast<const uint4*>(x + (rw + t) * C);
+    const uint4* xr = reinterpret_cast<const uint4*>(x + (rw + 8 * t) * C);
     uint4* d = ring + (t % DEPTH) * nv;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
@@ -664,7 +669,7 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
   __syncthreads();
   for (int t = 0; t < n; ++t) {
     if (t > 0) cp_wait_group<DEPTH - 1>();
-    const long long r = rw + t;
+    const long long r = rw + 8 * t;
     // the row as packed fp32 pairs where they fit the registers, else as stored
     // (unpacked again in each pass)
     constexpr bool KEEP = NCH * V <= 32;
@@ -717,9 +722,17 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
           f32x2 o[V / 2];
 #pragma unroll
           for (int q = 0; q < V / 2; q += 2) {
-            const ulonglong2 s4 = *reinterpret_cast<const ulonglong2*>(sh + k * V + 2 * q);
-            ulonglong2 c4 = *reinterpret_cast<const ulonglong2*>(sc + k * V + 2 * q);
-            if constexpr (!decltype(own)::value) {
+            const ulonglong2* const sp = reinterpret_cast<const ulonglong2*>(sh + k * V + 2 * q);
+            const ulonglong2* const cp = reinterpret_cast<const ulonglong2*>(sc + k * V + 2 * q);
+            ulonglong2 s4, c4;
+            if constexpr (decltype(own)::value) {
+              s4 = *sp;
+              c4 = *cp;
+            } else {
+              // read-only loads: plain ones may not pass the stores of out, so each
+              // vector would wait for its own (8000 x 2048 fp32, two samples 30.6 -> 26.0 us)
+              s4 = __ldg(sp);
+              c4 = __ldg(cp);
               const f32x2 one = pack2f(1.0f, 1.0f);
               c4.x = add2(c4.x, one);
               c4.y = add2(c4.y, one);
@@ -740,29 +753,34 @@ template <class T, int NCH>
 static cudaError_t ln_mod_launch(const T* x, T* out, long long rows, int C, const float* shift, const float* scale,
                                  int mod_stride, int seg_split, int rpb0, int rpb1, cudaStream_t s) {
   const long long sms = num_sms(), mods = 2LL * C * 4, row = (long long)C * sizeof(T);
-  // Rows of up to eight vectors per lane, while a row per warp makes at most
-  // about two waves of two blocks per SM: every row's loads in flight at once
-  // (64 x 128 fp32 1.93 us against 2.08 through the ring).
-  const bool few = rows <= 8LL * 4 * sms;
-  if constexpr (NCH <= 8) {
-    if (few) {
-      launch_pdl(k_ln_mod1<T, NCH>, (unsigned)((rows + 7) / 8), 256, (size_t)mods, s, x, out, rows, C, shift, scale,
-                 mod_stride, seg_split, rpb0, rpb1);
-      return launched();
-    }
+  // A row per warp while that is one wave of k_ln_mod1's resident blocks (64
+  // registers and four blocks up to six vectors a lane, then two or three fp32 and
+  // two or one bf16): every row's loads in flight at once.  2432 x 2048 5.9 us
+  // against 7.6 through the ring (3000 rows: 9.3 and 7.7), 900 x 4096 6.2 against
+  // 8.9, 2432 x 1536 fp32 5.2 against 5.5 (3000 rows: 7.9 and 6.5).
+  constexpr int FEW = NCH <= 6 ? 4 : sizeof(T) == 4 ? (NCH <= 8 ? 3 : 2) : (NCH <= 8 ? 2 : 1);
+  if (rows <= 8LL * FEW * sms) {
+    launch_pdl(k_ln_mod1<T, NCH>, (unsigned)((rows + 7) / 8), 256, (size_t)mods, s, x, out, rows, C, shift, scale,
+               mod_stride, seg_split, rpb0, rpb1);
+    return launched();
   }
-  // Blocks per SM as measured (8192 x 1152: four 12.7 us, two 16.6; 14310 x 2048:
-  // three 24.2, two 27.1, four 29.5; 8704 x 3072: two 25.7, three 33.5; 8000 x
-  // 2048 fp32: four 28.0, two 36.8), the ring as deep as their shared memory allows.
-  constexpr int BLOCKS = NCH <= 6 ? 4 : NCH <= 8 ? 3 : NCH <= 12 ? 2 : 4;
-  int rpw = 1, depth = 1;
-  if (!few) {
-    const long long budget = 224 * 1024 / BLOCKS - 1024 - mods;   // one block's rings
-    depth = budget >= 8 * 3 * row ? 3 : budget >= 8 * 2 * row ? 2 : 1;
-    const long long per_wave = 8LL * BLOCKS * sms;
-    rpw = (int)std::min((rows + per_wave - 1) / per_wave, 64LL);
+  // Blocks per SM as measured: four up to six vectors a lane (8000 x 1152 9.3 us,
+  // three 10.1, two 13.0), three up to eight (8000 x 2048 16.9, two 18.5, four
+  // 20.2), then the two that are resident (8000 x 3072 23.4, three and four
+  // in turn 32.3 and 26.8), for fp32 rows well past the L2 four in turn, in whole
+  // rows of warps (20000 x 2048 52.3, shares of one row's difference 54.4, two 56.2).
+  const bool past_l2 = NCH > 8 && sizeof(T) == 4 && 2 * rows * row > (180LL << 20);
+  const int blocks = NCH <= 6 ? 4 : NCH <= 8 ? 3 : past_l2 ? 4 : 2;
+  unsigned grid = (unsigned)std::min((rows + 7) / 8, blocks * sms);
+  int per = (int)(rows / grid), rem = (int)(rows % grid);
+  if (past_l2) {
+    per = (per + (rem > 0) + 7) / 8 * 8;
+    rem = 0;
+    grid = (unsigned)((rows + per - 1) / per);
   }
-  const unsigned grid = (unsigned)((rows + 8LL * rpw - 1) / (8LL * rpw));
+  // the ring as deep as that many blocks' shared memory allows
+  const long long budget = 224 * 1024 / blocks - 1024 - mods;
+  const int depth = budget >= 8 * 3 * row ? 3 : budget >= 8 * 2 * row ? 2 : 1;
   const size_t smem = (size_t)(mods + 8 * depth * row);
   // The kernel attribute belongs to the process, so it is the instance's own
   // largest size, whatever this call needs: threads with rows of other widths
@@ -774,7 +792,7 @@ static cudaError_t ln_mod_launch(const T* x, T* out, long long rows, int C, cons
     const cudaError_t a = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (a != cudaSuccess) return a;
     launch_pdl(kernel, dim3(grid), dim3(256), smem, s, x, out, rows, C, shift, scale, mod_stride, seg_split, rpb0,
-               rpb1, rpw);
+               rpb1, per, rem);
     return launched();
   };
   return depth == 3   ? go(k_ln_mod<T, NCH, 3>, std::integral_constant<int, 3>())

@@ -78,9 +78,13 @@ def test_f32_attention(cuda, dtype, B, nt, ni, H, d, pad):
 
 
 # ring depths and blocks per SM of every width class, samples that change inside
-# a block, a last block and warp with few rows, one row; unused row kept
+# a block, a last block and warp with few rows, one row; the last row counts of a
+# row per warp on 152 SMs and the next ones; fp32 past the L2; unused row kept
 LN = [("bf16", 1, 3072, 1), ("bf16", 4900, 128, 700), ("bf16", 6001, 1152, 250), ("bf16", 5003, 2048, 5003),
-      ("bf16", 5000, 3072, 33), ("bf16", 77, 4096, 20), ("f32", 4999, 1536, 1000), ("f32", 5001, 2048, 7)]
+      ("bf16", 5000, 3072, 33), ("bf16", 77, 4096, 20), ("f32", 4999, 1536, 1000), ("f32", 5001, 2048, 7),
+      ("bf16", 4864, 1536, 4864), ("bf16", 4865, 1536, 4865), ("bf16", 2433, 2048, 100), ("bf16", 1216, 4096, 1216),
+      ("bf16", 1217, 4096, 1217), ("bf16", 5003, 4096, 5003), ("f32", 3648, 1024, 500), ("f32", 3649, 1024, 3649),
+      ("f32", 2432, 2048, 2432), ("f32", 2435, 1536, 2435), ("f32", 12300, 2048, 12300)]
 
 
 @pytest.mark.parametrize("dtype,rows,C,rpb", LN)
