@@ -78,7 +78,10 @@ template <int BM_, int BN_, int TM_, int TN_, int WK_, int BK_, int ST_> struct 
   static_assert((BK / 4) % WK == 0, "every group takes whole 16-byte columns");
 };
 
-template <class C, bool VEC>
+// TAIL: the last stage is not a whole one and only its columns of K are copied and
+// multiplied (64 and 128 tiles; an instance of its own, because the loop over
+// columns costs the whole stages 1%): 4096 x 1152 x 16 22 -> 14 us.
+template <class C, bool VEC, bool TAIL>
 __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, const float* __restrict__ A, int lda,
                                                          const float* __restrict__ W, int ldw,
                                                          const __grid_constant__ EpiArgs e) {
@@ -114,11 +117,13 @@ __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, co
   for (int q = 0; q < PA; ++q) live |= (Mask)(m0 + r0 + RPP * q < M ? 1 : 0) << q;
 #pragma unroll
   for (int q = 0; q < PW; ++q) live |= (Mask)(n0 + r0 + RPP * q < N ? 1 : 0) << (PA + q);
+  const int K4 = (K + 3) & ~3;
   const float* const At = A + (size_t)m0 * lda;
   const float* const Wt = W + (size_t)n0 * ldw;
   auto load = [&](int kt, int slot) {
     float* s = sm + slot * C::STAGE + r0 * C::LD + kc;
     const int k0 = kt * C::BK;
+    if (TAIL && k0 + kc >= K4) return;                 // a column that is never read
     const Mask mask = k0 + kc < K ? live : (Mask)0;
 #pragma unroll
     for (int q = 0; q < PA + PW; ++q) {
@@ -143,31 +148,39 @@ __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, co
     if (kt0 + p < kt1) load(kt0 + p, p);
     cp_commit();
   }
-  for (int kt = kt0; kt < kt1; ++kt) {
+  // 16-byte column kk / 4 of stage `it`
+  auto column = [&](int it, int kk) {
+    const float* sa = sm + (it % C::ST) * C::STAGE + ra * C::LD + kk;
+    const float* sb = sm + (it % C::ST) * C::STAGE + (C::BM + rb) * C::LD + kk;
+    ulonglong2 a[C::TM], b[C::TN];
+#pragma unroll
+    for (int i = 0; i < C::TM; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(sa + 8 * i * C::LD);
+#pragma unroll
+    for (int j = 0; j < C::TN; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(sb + 4 * j * C::LD);
+#pragma unroll
+    for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+      for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].x, b[j].x);
+#pragma unroll
+    for (int i = 0; i < C::TM; ++i)
+#pragma unroll
+      for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].y, b[j].y);
+  };
+  const int full = TAIL ? min(kt1, K4 / C::BK) : kt1;  // whole stages [kt0, full)
+  for (int kt = kt0; kt < full; ++kt) {
     cp_wait<C::ST - 2>();
     __syncthreads();
     const int it = kt - kt0;
     if (kt + C::ST - 1 < kt1) load(kt + C::ST - 1, (it + C::ST - 1) % C::ST);
     cp_commit();
-    const float* sa = sm + (it % C::ST) * C::STAGE + ra * C::LD;
-    const float* sb = sm + (it % C::ST) * C::STAGE + (C::BM + rb) * C::LD;
 #pragma unroll
-    for (int c = 0; c < C::BK / 4 / C::WK; ++c) {
-      const int kk = (c * C::WK + wk) * 4;
-      ulonglong2 a[C::TM], b[C::TN];
-#pragma unroll
-      for (int i = 0; i < C::TM; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(sa + 8 * i * C::LD + kk);
-#pragma unroll
-      for (int j = 0; j < C::TN; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(sb + 4 * j * C::LD + kk);
-#pragma unroll
-      for (int i = 0; i < C::TM; ++i)
-#pragma unroll
-        for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].x, b[j].x);
-#pragma unroll
-      for (int i = 0; i < C::TM; ++i)
-#pragma unroll
-        for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].y, b[j].y);
-    }
+    for (int c = 0; c < C::BK / 4 / C::WK; ++c) column(it, (c * C::WK + wk) * 4);
+  }
+  if (TAIL && full < kt1) {
+    cp_wait<0>();
+    __syncthreads();
+#pragma unroll 1
+    for (int kk = wk * 4; kk < K4 - full * C::BK; kk += C::WK * 4) column(full - kt0, kk);
   }
   cp_wait<0>();
   __syncthreads();                                     // the stages are free: output tiles over them
@@ -267,11 +280,11 @@ __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, co
   cluster.sync();                                      // peers may still be reading this CTA's tile
 }
 
-template <class C, bool VEC>
-static cudaError_t gemm_f32_launch(int M, int N, int K, const float* A, int lda, const float* W, int ldw,
-                                   const EpiArgs& e, int split, cudaStream_t s) {
+template <class C, bool VEC, bool TAIL>
+static cudaError_t gemm_f32_tail(int M, int N, int K, const float* A, int lda, const float* W, int ldw,
+                                 const EpiArgs& e, int split, cudaStream_t s) {
   const cudaError_t attr =
-      cudaFuncSetAttribute(k_gemm_f32<C, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+      cudaFuncSetAttribute(k_gemm_f32<C, VEC, TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
   if (attr != cudaSuccess) return attr;
   const long long tiles = (long long)((N + C::BN - 1) / C::BN) * ((M + C::BM - 1) / C::BM);
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -289,13 +302,26 @@ static cudaError_t gemm_f32_launch(int M, int N, int K, const float* A, int lda,
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = split > 1 ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, k_gemm_f32<C, VEC>, M, N, K, A, lda, W, ldw, e);
+  cudaLaunchKernelEx(&cfg, k_gemm_f32<C, VEC, TAIL>, M, N, K, A, lda, W, ldw, e);
   return launched();
+}
+
+template <class C, bool VEC>
+static cudaError_t gemm_f32_launch(int M, int N, int K, const float* A, int lda, const float* W, int ldw,
+                                   const EpiArgs& e, int split, cudaStream_t s) {
+  if constexpr (C::BM >= 64)
+    if (K % C::BK != 0) return gemm_f32_tail<C, VEC, true>(M, N, K, A, lda, W, ldw, e, split, s);
+  return gemm_f32_tail<C, VEC, false>(M, N, K, A, lda, W, ldw, e, split, s);
 }
 
 // Tile choice by the estimated time of the launch's waves (one 128 or 64 tile
 // per SM at a time; a 64 tile's FMA count at 0.9 of the 128 tile's rate, a 32
-// tile's at 0.6).  Few rows or few tiles are latency- or weight-bound: 16 x 32
+// tile's at 0.6), then a smaller tile (never a larger one: smaller tiles have
+// more groups and so more partial sums, and short reductions should not lose
+// accuracy) where that is faster with what a tile takes beside its columns
+// of K counted in: 5.2, 2.7 and 0.53 us for the 128, 64 and 32 tiles, the time of
+// 56, 90 and 58 columns (657 x 1264 x 256 19.9 us in 64 tiles, 18.3 in 32).
+// Few rows or few tiles are latency- or weight-bound: 16 x 32
 // tiles up to 16 rows (W read once per 16 rows: 2 x 6912 x 1152 22.7 -> 15.2
 // us) and wherever 32 x 32 tiles would leave half the SMs idle (64 x 512 x 128
 // 3.46 -> 2.86 us); those also split K over a cluster while every CTA keeps a
@@ -313,11 +339,14 @@ static cudaError_t gemm_f32_t(int M, int N, int K, const float* A, int lda, cons
   const long long t64 = (long long)((M + 63) / 64) * ((N + 63) / 64);
   const long long t32 = (long long)((M + 31) / 32) * ((N + 31) / 32);
   if (M > 16 && t32 * 2 > sms) {
-    const double c128 = (double)((t128 + sms - 1) / sms) * 128 * 128;
-    const double c64 = (double)((t64 + sms - 1) / sms) * 64 * 64 * 1.1;
-    const double c32 = std::max(1.0, (double)t32 / sms) * 32 * 32 * 1.6;
-    if (c128 <= c64 && c128 <= c32) return gemm_f32_launch<C128, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
-    if (c64 <= c32) return gemm_f32_launch<C64, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
+    const double w128 = (double)((t128 + sms - 1) / sms) * 128 * 128, w64 = (double)((t64 + sms - 1) / sms) * 64 * 64;
+    const double w32 = std::max(1.0, (double)t32 / sms) * 32 * 32;
+    const double c128 = w128 * (K + 56), c64 = w64 * 1.165 * (K + 90), c32 = w32 * 1.7 * ((K + C32::BK - 1) / C32::BK * C32::BK + 58);
+    int bm = w128 <= w64 * 1.1 && w128 <= w32 * 1.6 ? 128 : w64 * 1.1 <= w32 * 1.6 ? 64 : 32;
+    if (bm == 128 && std::min(c64, c32) < c128) bm = c64 <= c32 ? 64 : 32;
+    if (bm == 64 && c32 < c64) bm = 32;
+    if (bm == 128) return gemm_f32_launch<C128, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
+    if (bm == 64) return gemm_f32_launch<C64, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
     return gemm_f32_launch<C32, VEC>(M, N, K, A, lda, W, ldw, e, 1, s);
   }
   const long long t16 = (long long)((M + 15) / 16) * ((N + 31) / 32);

@@ -25,7 +25,7 @@ TOL = 1e-6
 # row
 F32_GEMM = [(1, 32, 64), (16, 32, 300), (17, 36, 68), (64, 128, 512), (64, 128, 1100), (31, 4, 258), (10, 512, 128),
             (65, 4100, 96), (130, 700, 70), (512, 1152, 200), (500, 3460, 36), (2000, 1540, 33), (1024, 4608, 68),
-            (1024, 4608, 65), (2, 6912, 1152)]
+            (1024, 4608, 65), (2, 6912, 1152), (1175, 1156, 516), (1175, 1156, 517)]
 
 
 @pytest.mark.parametrize("M,N,K", F32_GEMM)
