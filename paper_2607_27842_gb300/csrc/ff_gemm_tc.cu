@@ -13,7 +13,8 @@
 //               GELU / gate / residual / history epilogue, stores through
 //               swizzled shared-memory blocks and TMA (16-byte stores where
 //               the output does not allow it); with one tile per CTA the
-//               residual / history-base blocks arrive by TMA as well.
+//               residual / history-base blocks arrive by TMA as well and are
+//               replaced in place by the output (epi_single).
 // Two TMEM accumulators (2 * BN columns) let the epilogue of tile i overlap
 // the main loop of tile i + 1.  Every mbarrier wait is bounded: on timeout
 // the CTA raises a watchdog flag, stops issuing work and releases its TMEM.
@@ -23,8 +24,9 @@
 // tiles run at half rate.  With BN = 256 the columns past the last
 // full 256-wide tile are covered by swapped tiles: up to 128 rows of W as
 // the MMA's M side against 256 rows of A as its N side (the accumulator
-// holds the transposed block; the epilogue transposes it back through a
-// 16 x 32 shared-memory buffer per warp).  DiT-XL/2's N = 1152 layers then
+// holds the transposed block: epi_single reads and writes it column by column,
+// the other epilogues transpose it back through a 16 x 32 shared-memory
+// buffer per warp).  DiT-XL/2's N = 1152 layers then
 // run as 4 x 32 full tiles + 16 swapped tiles, one wave of 144 tiles.
 #include "ff_common.cuh"
 #include "ff_tc.cuh"
@@ -64,15 +66,14 @@ __device__ __forceinline__ bool mbar_wait_u(uint64_t* b, uint32_t parity, volati
 }
 
 template <int BN> struct Cfg {
-  static constexpr int STAGES = BN >= 256 ? 4 : 6;
+  static constexpr int STAGES = 4;
   static constexpr uint32_t A_BYTES = BM * BK * 2;
   static constexpr uint32_t B_BYTES = BN * BK * 2;
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr uint32_t TMEM_COLS = 2 * BN;
-  // BN = 256 only: 4 KB per epilogue warp, two 32 x 32 bf16 output blocks
-  // for the TMA-store epilogue, or the 16 x 32 fp32 transpose buffer of a
-  // swapped tile
-  static constexpr uint32_t XPOSE_BYTES = BN >= 256 ? 8 * 4096 : 0;
+  // 4 KB per epilogue warp: two 32 x 32 bf16 output blocks for the TMA-store
+  // epilogues, or the 16 x 32 fp32 transpose buffer of a swapped tile
+  static constexpr uint32_t XPOSE_BYTES = 8 * 4096;
   static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + XPOSE_BYTES + 256;
   // instruction descriptor, kind::f16: D fp32 (bit 4), A bf16 (bits 7-9 = 1),
   // B bf16 (bits 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
@@ -81,7 +82,8 @@ template <int BN> struct Cfg {
 };
 
 // Tile list of one launch: n_norm normal tiles (128 rows of A x BN rows of
-// W, M-fastest), then swapped tiles (128 rows of W x 256 rows of A).
+// W, in the order of grouped_tile), then swapped tiles (128 rows of W x 256
+// rows of A).
 struct TileMap {
   int num_m;   // 128-row blocks of A
   int n_full;  // BN-wide column blocks of the normal tiles
@@ -89,9 +91,10 @@ struct TileMap {
   int num_m2;  // 256-row blocks of A (swapped tiles)
   int n_tiles; // n_norm + swapped tiles
   int staged;  // normal tiles store out (and hist_out) through shared memory + TMA
-  // one tile per CTA (the TMA ring is idle after its mainloop): each
-  // epilogue warp loads its residual (bit 0) and history-base (bit 1) block
-  // with TMA into the freed ring instead of per-lane global loads
+  // one tile per CTA: the residual (bit 0) and the history base (bit 1) can be
+  // described by a tensor map.  epi_single takes them so; the shared epilogue
+  // loads them with TMA into the ring, idle after its mainloop, where the
+  // LayerNorm is fused (its other instances load them per lane)
   int pre;
 };
 
@@ -165,9 +168,8 @@ enum { EPI_FULL = 0, EPI_PLAIN = 1, EPI_SINGLE = 2, EPI_SINGLE_HIST = 3 };
 // parameter (a run-time choice between two parameter structs turns every
 // field access of the inner loops into a generic load).  PLAIN: normal
 // tiles without residual preloads (the second problem of a grouped launch,
-// the CTA pairs).  XB: bytes of the epilogue warps' staging buffers (0: the
-// per-lane store path only).  Returns false when the accumulator wait gave up.
-template <int BN, int XB, bool PLAIN, int LN, int EPI>
+// the CTA pairs).  Returns false when the accumulator wait gave up.
+template <int BN, bool PLAIN, int LN, int EPI>
 __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, const TileMap& tm, const int M,
                                          const int N, const TileAt t, const int acc, const uint32_t aph,
                                          uint32_t& epi_cnt, const CUtensorMap* tmO, const CUtensorMap* tmH,
@@ -232,7 +234,7 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
       }
     }
   };
-  if (XB > 0 && tm.staged && !sw) {
+  if (tm.staged && !sw) {
     if constexpr (EPI == EPI_PLAIN) fetch_bias(t.n0 + c_lo); else fetch(t.n0 + c_lo);
   }
   int ok = 1;
@@ -265,7 +267,7 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
     return __shfl_sync(0xffffffffu, w, 0) != 0;
   };
   const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
-  if (!sw && (XB == 0 || !tm.staged)) {
+  if (!sw && !tm.staged) {
     const int m = t.m0 + row;
     const float2 lnr = ((LN == 1 && e.ln_in) && m < M) ? ln_row(e, m) : make_float2(1.f, 0.f);
     for (int c = h * (BN / 2); c < (h + 1) * (BN / 2); c += 32) {
@@ -426,7 +428,7 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
       }
       ++epi_cnt;
     }
-  } else if constexpr (XB > 0) {
+  } else {
     // lane = output column n + lane; TMEM column = output row.  Blocks of
     // 16 rows x 32 columns go through the warp's buffer (XOR-swizzled,
     // conflict-free both ways); afterwards lane l holds row l / 2,
@@ -910,19 +912,19 @@ __global__ void __launch_bounds__(THREADS, 1)
       if constexpr (EPI == EPI_SINGLE || EPI == EPI_SINGLE_HIST) {
         ok = epi_single<BN, EPI == EPI_SINGLE>(W, e0, M0, N, tile_at<BN>(tm0, tile), &tmO, &tmH, &tmR, &tmHB);
       } else if constexpr (GROUPED) {
-        ok = tile < n1 ? epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN, EPI>(W, e1, tm1, M1, N, tile_at<BN>(tm1, tile), acc, aph, epi_cnt, &tmO1,
+        ok = tile < n1 ? epi_tile<BN, true, LN, EPI>(W, e1, tm1, M1, N, tile_at<BN>(tm1, tile), acc, aph, epi_cnt, &tmO1,
                                             &tmH1, &tmR, &tmHB)
-                       : epi_tile<BN, Cfg<BN>::XPOSE_BYTES, true, LN, EPI>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile - n1), acc, aph, epi_cnt, &tmO,
+                       : epi_tile<BN, true, LN, EPI>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile - n1), acc, aph, epi_cnt, &tmO,
                                             &tmH, &tmR, &tmHB);
       } else {
-        ok = epi_tile<BN, Cfg<BN>::XPOSE_BYTES, false, LN, EPI>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile), acc, aph, epi_cnt, &tmO, &tmH, &tmR,
+        ok = epi_tile<BN, false, LN, EPI>(W, e0, tm0, M0, N, tile_at<BN>(tm0, tile), acc, aph, epi_cnt, &tmO, &tmH, &tmR,
                                  &tmHB);
       }
       if (!ok) break;
       tc_fence_before();
       mbar_arrive(&tempty[acc]);
     }
-    if (C::XPOSE_BYTES > 0 && lane == 0) bulk_wait_all();  // TMA stores complete before exit
+    if (lane == 0) bulk_wait_all();  // TMA stores complete before exit
   }
   tc_fence_before();
   __syncthreads();
@@ -1113,10 +1115,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       const TileAt t = {false, mb * 2 * BM + (int)rank * BM, nb * BN};
       bool ok;
       if (g1)
-        ok = epi_tile<BN, C::XPOSE_BYTES, true, LN, EPI>(W, e1, tm1, M1, N, t, acc, aph, epi_cnt, &tmO1, &tmH1, &tmO1,
+        ok = epi_tile<BN, true, LN, EPI>(W, e1, tm1, M1, N, t, acc, aph, epi_cnt, &tmO1, &tmH1, &tmO1,
                                                      &tmO1);
       else
-        ok = epi_tile<BN, C::XPOSE_BYTES, true, LN, EPI>(W, e, tm, M, N, t, acc, aph, epi_cnt, &tmO, &tmH, &tmO, &tmO);
+        ok = epi_tile<BN, true, LN, EPI>(W, e, tm, M, N, t, acc, aph, epi_cnt, &tmO, &tmH, &tmO, &tmO);
       if (!ok) break;
       tc_fence_before();
       mbar_arrive_cluster(map_to(&tempty[acc], 0));
@@ -1142,12 +1144,10 @@ template <int BN, bool G>
 auto gemm_fn(int ln, int epi) -> decltype(&k_gemm_tc<BN, G, 0, EPI_FULL>) {
   if (ln == 1) return k_gemm_tc<BN, G, 1, EPI_FULL>;
   if (ln == 2) return k_gemm_tc<BN, G, 2, EPI_FULL>;
-  if constexpr (BN == 256) {
-    if (epi == EPI_PLAIN) return k_gemm_tc<BN, G, 0, EPI_PLAIN>;
-    if constexpr (!G) {
-      if (epi == EPI_SINGLE) return k_gemm_tc<BN, G, 0, EPI_SINGLE>;
-      if (epi == EPI_SINGLE_HIST) return k_gemm_tc<BN, G, 0, EPI_SINGLE_HIST>;
-    }
+  if (epi == EPI_PLAIN) return k_gemm_tc<BN, G, 0, EPI_PLAIN>;
+  if constexpr (!G) {
+    if (epi == EPI_SINGLE) return k_gemm_tc<BN, G, 0, EPI_SINGLE>;
+    if (epi == EPI_SINGLE_HIST) return k_gemm_tc<BN, G, 0, EPI_SINGLE_HIST>;
   }
   return k_gemm_tc<BN, G, 0, EPI_FULL>;
 }
@@ -1194,7 +1194,6 @@ bool init_driver() {
     };
     for (int ln = 0; ln < 3; ++ln)
       for (int epi : {EPI_FULL, EPI_PLAIN, EPI_SINGLE, EPI_SINGLE_HIST}) {
-        smem((const void*)gemm_fn<128, false>(ln, epi), Cfg<128>::SMEM);
         smem((const void*)gemm_fn<256, false>(ln, epi), Cfg<256>::SMEM);
         smem((const void*)gemm_fn<256, true>(ln, epi), Cfg<256>::SMEM);
         smem((const void*)gemm2_fn<128>(ln, epi), Cfg2<128>::SMEM);
@@ -1305,50 +1304,35 @@ cudaError_t gemm_tc(int M, int N, int K, const void* A, int lda, const void* W, 
                  mo, mh, 0, none, e);
     return launched();
   }
-  // Every tile (128 x 256 full rate, 128 x 128 at half rate, swapped 128 x
-  // 256) takes about the same time: take the tiling with the fewest waves,
-  // ties to full-rate tiles.
+  // 128 x 256 tiles, remainder columns in swapped tiles (128-wide tiles would run
+  // at half rate and be as many at least)
   TileMap tm;
+  const int rem = N % 256;
+  const long long tiles = wide_tiles(M, N);
   tm.num_m = (M + BM - 1) / BM;
   tm.num_m2 = (M + 255) / 256;
-  const int rem = N % 256;
-  const long long t256 = wide_tiles(M, N);
-  const long long t128 = (long long)tm.num_m * ((N + 127) / 128);
-  const bool wide = (t256 + g_sms - 1) / g_sms <= (t128 + g_sms - 1) / g_sms;
-  CUtensorMap mw128 = {}, ma256 = {}, mo = {}, mh = {}, mr = {}, mhb = {};
-  tm.staged = 0;
+  tm.n_full = N / 256;
+  tm.n_norm = tm.num_m * tm.n_full;
+  tm.n_tiles = (int)tiles;
   tm.pre = 0;
-  if (wide) {
-    tm.n_full = N / 256;
-    tm.n_norm = tm.num_m * tm.n_full;
-    tm.n_tiles = (int)t256;
-    if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, 256)) return cudaErrorInvalidValue;
-    if (rem && (!make_map(&mw128, W, N, K, ldw, BM) || !make_map(&ma256, A, M, K, lda, 256)))
-      return cudaErrorInvalidValue;
-    tm.staged = staged_maps(e, M, N, &mo, &mh) ? 1 : 0;
-    // one tile per CTA: residual / history-base blocks by TMA (16-byte aligned
-    // rows; otherwise the per-lane loads stay)
-    int epi = epi_form(e);
-    if (tm.staged && t256 <= g_sms) {
-      if (e.resid && make_store_map(&mr, const_cast<void*>(e.resid), M, N, e.ld_resid)) tm.pre |= 1;
-      if (e.hist_out && make_store_map(&mhb, const_cast<void*>(e.hist_base), M, N, e.ldo)) tm.pre |= 2;
-      const bool blocks = (!e.resid || (tm.pre & 1)) && (!e.hist_out || (tm.pre & 2)) && tm.pre;
-      if (blocks && !e.rope && e.act != 2 && e.act_col0 == 0) epi = e.resid ? EPI_SINGLE : EPI_SINGLE_HIST;
-    }
-    const int grid = (int)(t256 < g_sms ? t256 : g_sms);
-    const TileMap none = {};
-    launch_pdl(gemm_fn<256, false>(ln_side(e), epi), grid, THREADS, Cfg<256>::SMEM, s, ma, mb, mw128, ma256, mo, mh, mr, mhb, M, N, K, tm,
-               e, ma, mb, mo, mh, 0, none, e);
-  } else {
-    tm.n_full = (N + 127) / 128;
-    tm.n_norm = tm.num_m * tm.n_full;
-    tm.n_tiles = tm.n_norm;
-    if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, 128)) return cudaErrorInvalidValue;
-    const int grid = (int)(t128 < g_sms ? t128 : g_sms);
-    const TileMap none = {};
-    launch_pdl(gemm_fn<128, false>(ln_side(e), EPI_FULL), grid, THREADS, Cfg<128>::SMEM, s, ma, mb, ma, mb, ma, mb, ma, mb, M, N, K, tm, e, ma,
-               mb, ma, mb, 0, none, e);
+  CUtensorMap mw128 = {}, ma256 = {}, mo = {}, mh = {}, mr = {}, mhb = {};
+  if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, W, N, K, ldw, 256)) return cudaErrorInvalidValue;
+  if (rem && (!make_map(&mw128, W, N, K, ldw, BM) || !make_map(&ma256, A, M, K, lda, 256)))
+    return cudaErrorInvalidValue;
+  tm.staged = staged_maps(e, M, N, &mo, &mh) ? 1 : 0;
+  // one tile per CTA: residual / history-base blocks by TMA (16-byte aligned
+  // rows; otherwise the per-lane loads stay)
+  int epi = epi_form(e);
+  if (tm.staged && tiles <= g_sms) {
+    if (e.resid && make_store_map(&mr, const_cast<void*>(e.resid), M, N, e.ld_resid)) tm.pre |= 1;
+    if (e.hist_out && make_store_map(&mhb, const_cast<void*>(e.hist_base), M, N, e.ldo)) tm.pre |= 2;
+    const bool blocks = (!e.resid || (tm.pre & 1)) && (!e.hist_out || (tm.pre & 2)) && tm.pre;
+    if (blocks && !e.rope && e.act != 2 && e.act_col0 == 0) epi = e.resid ? EPI_SINGLE : EPI_SINGLE_HIST;
   }
+  const int grid = (int)(tiles < g_sms ? tiles : g_sms);
+  const TileMap none = {};
+  launch_pdl(gemm_fn<256, false>(ln_side(e), epi), grid, THREADS, Cfg<256>::SMEM, s, ma, mb, mw128, ma256, mo, mh, mr, mhb, M, N, K, tm,
+             e, ma, mb, mo, mh, 0, none, e);
   return launched();
 }
 
