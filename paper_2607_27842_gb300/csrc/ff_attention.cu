@@ -19,11 +19,6 @@ namespace {
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr(dst)), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -112,7 +107,7 @@ __global__ void __launch_bounds__(128) k_attn_mma(AttnArgs a, float scale_log2) 
   };
   load_kv(0, 0);
   cp_commit();
-  cp_wait_all();
+  cp_wait<0>();
   __syncthreads();
 
   uint32_t qf[DK / 16][4];
@@ -218,7 +213,7 @@ __global__ void __launch_bounds__(128) k_attn_mma(AttnArgs a, float scale_log2) 
         mma16816(o[NTD - 1], pa, r[0], r[1]);
       }
     }
-    cp_wait_all();
+    cp_wait<0>();
     __syncthreads();
   }
 

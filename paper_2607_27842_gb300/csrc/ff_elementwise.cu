@@ -566,37 +566,6 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : 1) k_ln_mod1(const T* __re
 // 3072 38.4, 25.8, 24.3; 4608 x 3072 22.2, 18.7, 15.1; 8000 x 2048 17.9, 19.1, 16.7;
 // 8192 x 1152 15.2, 10.3, 9.3; 14000 x 128 9.5, 5.1, 5.1; 14310 x 2048 24.9, 24.5,
 // 24.2 (4.8 TB/s).
-__device__ __forceinline__ void cp16_async(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// packed fp32 pairs (fma.rn.f32x2: two results an instruction)
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2f(float a, float b) {
-  return (f32x2)__float_as_uint(a) | ((f32x2)__float_as_uint(b) << 32);
-}
-__device__ __forceinline__ float lo2(f32x2 x) { return __uint_as_float((unsigned)x); }
-__device__ __forceinline__ float hi2(f32x2 x) { return __uint_as_float((unsigned)(x >> 32)); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 // a 16-byte vector of four fp32 or eight bf16 values <-> pairs
 __device__ __forceinline__ void unpack2x(const uint4& v, f32x2 (&p)[2]) {
   p[0] = (f32x2)v.x | ((f32x2)v.y << 32);
@@ -605,7 +574,7 @@ __device__ __forceinline__ void unpack2x(const uint4& v, f32x2 (&p)[2]) {
 __device__ __forceinline__ void unpack2x(const uint4& v, f32x2 (&p)[4]) {
   const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int i = 0; i < 4; ++i) p[i] = (f32x2)(w[i] << 16) | ((f32x2)(w[i] & 0xffff0000u) << 32);
+  for (int i = 0; i < 4; ++i) p[i] = bf2u(w[i]);
 }
 __device__ __forceinline__ uint4 packv(const f32x2 (&o)[2]) {
   return make_uint4((unsigned)o[0], (unsigned)(o[0] >> 32), (unsigned)o[1], (unsigned)(o[1] >> 32));
@@ -614,7 +583,7 @@ __device__ __forceinline__ uint4 packv(const f32x2 (&o)[4]) {
   uint32_t w[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(lo2(o[i]), hi2(o[i]));
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo_f(o[i]), hi_f(o[i]));
     w[i] = *reinterpret_cast<const uint32_t*>(&h);
   }
   return make_uint4(w[0], w[1], w[2], w[3]);
@@ -644,7 +613,7 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
       const int k = lane + 32 * j;
-      if (k < nv) cp16_async(d + k, xr + k);
+      if (k < nv) cp_async16(d + k, xr + k);
     }
   };
 #pragma unroll
@@ -654,13 +623,13 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
       const float4* sh4 = reinterpret_cast<const float4*>(shift + (size_t)b0 * mod_stride);
       const float4* sc4 = reinterpret_cast<const float4*>(scale + (size_t)b0 * mod_stride);
       for (int i = threadIdx.x; i < C / 4; i += blockDim.x) {
-        cp16_async(smod4 + i, sh4 + i);
-        cp16_async(smod4 + C / 4 + i, sc4 + i);
+        cp_async16(smod4 + i, sh4 + i);
+        cp_async16(smod4 + C / 4 + i, sc4 + i);
       }
     }
-    cp_commit_group();
+    cp_commit();
   }
-  cp_wait_group<DEPTH - 1>();
+  cp_wait<DEPTH - 1>();
   for (int i = threadIdx.x; i < C / 4; i += blockDim.x) {   // 1 + scale, each thread its own copies
     float4 v = smod4[C / 4 + i];
     v.x += 1.0f; v.y += 1.0f; v.z += 1.0f; v.w += 1.0f;
@@ -668,7 +637,7 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
   }
   __syncthreads();
   for (int t = 0; t < n; ++t) {
-    if (t > 0) cp_wait_group<DEPTH - 1>();
+    if (t > 0) cp_wait<DEPTH - 1>();
     const long long r = rw + 8 * t;
     // the row as packed fp32 pairs where they fit the registers, else as stored
     // (unpacked again in each pass)
@@ -685,13 +654,13 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
         f32x2 (&p)[V / 2] = a[KEEP ? j : 0];
         unpack2x(v, p);
 #pragma unroll
-        for (int q = 0; q < V / 2; ++q) s2 = add2(s2, p[q]);
+        for (int q = 0; q < V / 2; ++q) s2 = fadd2(s2, p[q]);
       }
     }
-    const float mean = warp_sum(lo2(s2) + hi2(s2)) / C;
+    const float mean = warp_sum(lo_f(s2) + hi_f(s2)) / C;
     if (t + DEPTH < n) copy_row(t + DEPTH);          // the slot has been read (its values are in the sum)
-    cp_commit_group();
-    const f32x2 nm = pack2f(-mean, -mean);
+    cp_commit();
+    const f32x2 nm = f2u(-mean, -mean);
     f32x2 ss2 = 0ull;
 #pragma unroll
     for (int j = 0; j < NCH; ++j) {
@@ -700,14 +669,14 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
         if constexpr (!KEEP) unpack2x(cur[j], p);
 #pragma unroll
         for (int q = 0; q < V / 2; ++q) {
-          const f32x2 d = add2(p[q], nm);
+          const f32x2 d = fadd2(p[q], nm);
           if constexpr (KEEP) p[q] = d;              // centred from here on
-          ss2 = fma2(d, d, ss2);
+          ss2 = ffma2(d, d, ss2);
         }
       }
     }
-    const float rstd = rsqrtf(warp_sum(lo2(ss2) + hi2(ss2)) / C + 1e-6f);
-    const f32x2 rs = pack2f(rstd, rstd);
+    const float rstd = rsqrtf(warp_sum(lo_f(ss2) + hi_f(ss2)) / C + 1e-6f);
+    const f32x2 rs = f2u(rstd, rstd);
     const int b = (int)(r < seg_split ? r / rpb0 : (r - seg_split) / rpb1);
     uint4* const orow = reinterpret_cast<uint4*>(out + r * C);
     // the block's sample from shared memory (scale already 1 + scale), another
@@ -733,12 +702,12 @@ __global__ void __launch_bounds__(256, NCH <= 6 ? 4 : NCH <= 8 ? 3 : 2)
               // vector would wait for its own (8000 x 2048 fp32, two samples 30.6 -> 26.0 us)
               s4 = __ldg(sp);
               c4 = __ldg(cp);
-              const f32x2 one = pack2f(1.0f, 1.0f);
-              c4.x = add2(c4.x, one);
-              c4.y = add2(c4.y, one);
+              const f32x2 one = f2u(1.0f, 1.0f);
+              c4.x = fadd2(c4.x, one);
+              c4.y = fadd2(c4.y, one);
             }
-            o[q] = fma2(mul2(KEEP ? p[q] : add2(p[q], nm), rs), c4.x, s4.x);
-            o[q + 1] = fma2(mul2(KEEP ? p[q + 1] : add2(p[q + 1], nm), rs), c4.y, s4.y);
+            o[q] = ffma2(fmul2(KEEP ? p[q] : fadd2(p[q], nm), rs), c4.x, s4.x);
+            o[q + 1] = ffma2(fmul2(KEEP ? p[q + 1] : fadd2(p[q + 1], nm), rs), c4.y, s4.y);
           }
           orow[k] = packv(o);
         }

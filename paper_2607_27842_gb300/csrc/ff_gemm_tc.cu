@@ -108,7 +108,7 @@ __device__ __forceinline__ float2 unpack2(uint32_t u) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
 }
 // gelu_tanh_fast on 16 packed pairs
-__device__ __forceinline__ void gelu_pairs(unsigned long long (&y)[16]) {
+__device__ __forceinline__ void gelu_pairs(f32x2 (&y)[16]) {
   const unsigned long long k0 = f2u(GELU_K0, GELU_K0), k1 = f2u(GELU_K1, GELU_K1), hf = f2u(0.5f, 0.5f);
 #pragma unroll
   for (int i = 0; i < 16; ++i) {

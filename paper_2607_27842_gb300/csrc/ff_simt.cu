@@ -48,22 +48,6 @@ static int sm_count() {
 // everywhere: 1024 x 4608 x 4608 1775 -> 870 us, 512 x 1152 x 4608 562 -> 131,
 // 64 x 128 x 512 60 -> 4.3, 2 x 6912 x 1152 122 -> 15.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp16(void* dst, const void* src, bool in) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(in ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp4(void* dst, const void* src, bool in) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(in ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void ffma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
-}
-
 // BM x BN tile, warp tile 8 TM x 4 TN (lanes 8 x 4), WK groups of warps
 template <int BM_, int BN_, int TM_, int TN_, int WK_, int BK_, int ST_> struct F32Cfg {
   static constexpr int BM = BM_, BN = BN_, TM = TM_, TN = TN_, WK = WK_, BK = BK_, ST = ST_;
@@ -132,11 +116,11 @@ __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, co
                                 : Wt + k0 + (ow + (Off)(RPP * (q - PA)) * (Off)ldw);
       src = in ? src : A;
       float* d = s + (q < PA ? RPP * q : C::BM + RPP * (q - PA)) * C::LD;
-      if (VEC) cp16(d, src, in); else cp4(d, src, in);
+      if (VEC) cp_async16(d, src, in ? 16 : 0); else cp_async4(d, src, in ? 4 : 0);
     }
   };
 
-  unsigned long long acc[C::TM][C::TN];
+  f32x2 acc[C::TM][C::TN];
 #pragma unroll
   for (int i = 0; i < C::TM; ++i)
 #pragma unroll
@@ -160,11 +144,11 @@ __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, co
 #pragma unroll
     for (int i = 0; i < C::TM; ++i)
 #pragma unroll
-      for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].x, b[j].x);
+      for (int j = 0; j < C::TN; ++j) acc[i][j] = ffma2(a[i].x, b[j].x, acc[i][j]);
 #pragma unroll
     for (int i = 0; i < C::TM; ++i)
 #pragma unroll
-      for (int j = 0; j < C::TN; ++j) ffma2(acc[i][j], a[i].y, b[j].y);
+      for (int j = 0; j < C::TN; ++j) acc[i][j] = ffma2(a[i].y, b[j].y, acc[i][j]);
   };
   const int full = TAIL ? min(kt1, K4 / C::BK) : kt1;  // whole stages [kt0, full)
   for (int kt = kt0; kt < full; ++kt) {
@@ -190,8 +174,7 @@ __global__ void __launch_bounds__(C::THREADS) k_gemm_f32(int M, int N, int K, co
     for (int i = 0; i < C::TM; ++i)
 #pragma unroll
       for (int j = 0; j < C::TN; ++j)
-        t[(ra + 8 * i) * C::LDC + rb + 4 * j] =
-            __uint_as_float((unsigned)acc[i][j]) + __uint_as_float((unsigned)(acc[i][j] >> 32));
+        t[(ra + 8 * i) * C::LDC + rb + 4 * j] = lo_f(acc[i][j]) + hi_f(acc[i][j]);
   }
   __syncthreads();
   // four consecutive columns of one row per thread: the groups' partials in
@@ -409,7 +392,7 @@ __global__ void __launch_bounds__(FA_THREADS) k_attn_f32(AttnArgs a, float scale
       const T* src = in ? g + tok_row(a, b, n0 + r) * a.ld_qkv + e : g;
       float* d = s + r * ld + e;
       if constexpr (VEC && sizeof(T) == 4) {
-        cp16(d, src, in);
+        cp_async16(d, src, in ? 16 : 0);
       } else if constexpr (VEC) {
         float v[VecN<T>::n];
         ld16(src, v);
@@ -442,7 +425,7 @@ __global__ void __launch_bounds__(FA_THREADS) k_attn_f32(AttnArgs a, float scale
   for (int t = 0; t < nt; ++t) {
     cp_wait<1>();                                      // this tile's keys (its values may be in flight)
     __syncthreads();
-    unsigned long long s2[4][4];
+    f32x2 s2[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -457,11 +440,11 @@ __global__ void __launch_bounds__(FA_THREADS) k_attn_f32(AttnArgs a, float scale
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ffma2(s2[i][j], qv[i].x, kv[j].x);
+        for (int j = 0; j < 4; ++j) s2[i][j] = ffma2(qv[i].x, kv[j].x, s2[i][j]);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ffma2(s2[i][j], qv[i].y, kv[j].y);
+        for (int j = 0; j < 4; ++j) s2[i][j] = ffma2(qv[i].y, kv[j].y, s2[i][j]);
     }
     __syncthreads();                                   // the key buffer is free
     if (t + 1 < nt) load(a.k, sK, (t + 1) * FA_BK, FA_BK);
@@ -471,7 +454,7 @@ __global__ void __launch_bounds__(FA_THREADS) k_attn_f32(AttnArgs a, float scale
       float s[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float dot = __uint_as_float((unsigned)s2[i][j]) + __uint_as_float((unsigned)(s2[i][j] >> 32));
+        const float dot = lo_f(s2[i][j]) + hi_f(s2[i][j]);
         s[j] = t * FA_BK + tk + 16 * j < N ? dot * scale : -INFINITY;
       }
       float cm = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
