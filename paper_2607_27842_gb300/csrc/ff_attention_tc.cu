@@ -28,10 +28,10 @@
 // tile's chain of S -> softmax -> P V, about 3700 cycles per key tile of
 // which the tile's own MMAs are 1650, the exponentials 1050 and the hand-offs
 // the rest; the MMAs alone (no softmax) take 861 us, the softmax alone about
-// as long.  Two threads per row instead of one (four softmax warps per
+// as long.  (Times here and below: launches back to back in a CUDA graph.)  Two threads per row instead of one (four softmax warps per
 // scheduler): 1324 -> 1260 us; every lane polling the S barrier instead of one
-// lane and a shuffle: 5%; one elected block per group of MMAs: 2%.  Now 1180
-// us (1470 TFLOP/s); 4096 + 512 tokens, 24 heads 226 -> 209 us.
+// lane and a shuffle: 5%; one elected block per group of MMAs: 2%.  Now 1160
+// us (1500 TFLOP/s); 4096 + 512 tokens, 24 heads 226 -> 204 us.
 // TMEM columns: S_0 [0,128), S_1 [128,256), O_0 [256,384), O_1 [384,512);
 // with one query tile per CTA (short sequences): S [0,128), O [128,256).  P of a
 // half tile lies over the start of that half's S columns.
@@ -693,8 +693,9 @@ __global__ void __launch_bounds__(ACfg<D, QT>::THREADS, QT == 1 ? 2 : 1)
 
 
 // ---------------------------------------------------------------------------
-// (16 x 256 tokens, 16 heads x 72: 17.6 -> 14.7 us with every lane polling, one
-// arrival per warp and one elected block per group of MMAs)
+// (16 x 256 tokens, 16 heads x 72: 16.0 -> 15.0 us with every lane polling, one
+// arrival per warp and one elected block per group of MMAs; a call by itself
+// 17.9 -> 16.5)
 // Sequences of at most two key tiles (256 tokens; DiT-XL/2) with a head
 // width of at most 80: one query tile at a time, two CTAs per SM, every CTA
 // taking the query tiles of one (sample, head) in turn.  The head's K and V

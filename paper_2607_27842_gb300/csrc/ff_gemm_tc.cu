@@ -15,6 +15,8 @@
 //               the output does not allow it); with one tile per CTA the
 //               residual / history-base blocks arrive by TMA as well and are
 //               replaced in place by the output (epi_single).
+// Times in the comments are of launches back to back in a CUDA graph.
+//
 // Two TMEM accumulators (2 * BN columns) let the epilogue of tile i overlap
 // the main loop of tile i + 1.  Every mbarrier wait is bounded: on timeout
 // the CTA raises a watchdog flag, stops issuing work and releases its TMEM.
@@ -124,7 +126,7 @@ struct TileAt {
 // its rows fastest, so the tiles running together cover about a square of the
 // output and a group's rows of A are read from DRAM once (with all row blocks
 // fastest, 14310 x 2048 x 8192 read its 234 MB of A for each of the 8 column
-// blocks: 1515 MB of DRAM traffic and 333 us, now 290 us).
+// blocks: 1515 MB of DRAM traffic and 322 us, now 291 us).
 template <int GM>
 __device__ __forceinline__ void grouped_tile(int tile, int num_m, int num_n, int& m, int& n) {
   const int g = tile / (GM * num_n), r = tile - g * GM * num_n;
@@ -283,8 +285,8 @@ __device__ __forceinline__ bool epi_tile(const EpiWarp& W, const EpiArgs& e, con
   } else if (EPI == EPI_PLAIN && !sw) {
     // Staged epilogue of a layer without gate, residual and history: as
     // below, in packed fp32 pairs and without shuffles (the costliest
-    // instructions beside a mainloop): 4096 x 4608 x 1152 with GELU 39.7 -> 33.6
-    // us, 14310 x 8192 x 2048 302 -> 273
+    // instructions beside a mainloop): on single CTAs, 4096 x 4608 x 1152 with
+    // GELU 39.7 -> 33.6 us, 14310 x 8192 x 2048 302 -> 273 (on pairs 30 and 254)
     const int m = t.m0 + row;
     for (int c = c_lo; c < c_lo + BN / 2; c += 32) {
       const int n0 = t.n0 + c;
@@ -580,7 +582,7 @@ __device__ __forceinline__ int sample_end(const EpiArgs& e, int r) {
 // 64-byte read and write, with no transposition buffer.
 // Against the shared form with its block-by-block buffers, shuffled bias and
 // gate and transposed swapped tiles: 4096 x 1152 x 1152 (gate, residual) 19.3
-// -> 14.5 us, 4096 x 1152 x 4608 (and history) 46.2 -> 41.0 us.
+// -> 14.5 us, 4096 x 1152 x 4608 (and history) 46.2 -> 40.1 us.
 template <int BN, bool RES>
 __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, const int M, const int N, const TileAt t,
                                            const CUtensorMap* tmO, const CUtensorMap* tmH, const CUtensorMap* tmR,
@@ -731,8 +733,8 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
       for (int j = 0; j < 32; ++j) v[j] *= j < jb ? c0[i] : c1[i];
       if ((hist || i >= 2) && !late_ready()) return false;
       // a pass of reads, then one of writes: alternating, every read would wait
-      // behind the write before it (37 x 48 x 1192, residual and history 13.6 -> 11.1 us,
-      // 4096 x 1152 x 4608 with gate, residual and history 43.0 -> 41.0)
+      // behind the write before it (37 x 48 x 1192, residual and history 13.6 -> 10.8 us,
+      // 4096 x 1152 x 4608 with gate, residual and history 43.0 -> 40.1)
       auto at = [&](uint8_t* blk, int j) { return reinterpret_cast<bf16*>(blk + j * 64 + off[(j >> 1) & 3]); };
       if constexpr (RES) {
 #pragma unroll

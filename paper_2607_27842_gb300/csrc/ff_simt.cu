@@ -38,7 +38,8 @@ static int sm_count() {
 // they add through distributed shared memory, rank by rank, so the result
 // does not depend on timing.
 //
-// Bound: FFMA2 issue beside the fragment loads.  A register-only FFMA2 loop
+// Bound (times: launches back to back in a CUDA graph): FFMA2 issue beside the
+// fragment loads.  A register-only FFMA2 loop
 // runs at 114 of the 128 FMA per SM and clock (scalar FFMA 76), with this
 // kernel's 16 16-byte loads per 256 FMA 91; the 128 tile reaches 83.  What
 // counted: deep stages (BK 32 -> 128 on 64 tiles: 512 x 1152 x 1152 42 -> 36
