@@ -729,8 +729,10 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = gelu_tanh_fast(v[j]);
       }
+      // (the gate's product rounded before the residual is added, as in the normal
+      // tiles: no contraction to an fma)
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] *= j < jb ? c0[i] : c1[i];
+      for (int j = 0; j < 32; ++j) v[j] = __fmul_rn(v[j], j < jb ? c0[i] : c1[i]);
       if ((hist || i >= 2) && !late_ready()) return false;
       // a pass of reads, then one of writes: alternating, every read would wait
       // behind the write before it (37 x 48 x 1192, residual and history 13.6 -> 10.8 us,
@@ -738,7 +740,7 @@ __device__ __forceinline__ bool epi_single(const EpiWarp& W, const EpiArgs& e, c
       auto at = [&](uint8_t* blk, int j) { return reinterpret_cast<bf16*>(blk + j * 64 + off[(j >> 1) & 3]); };
       if constexpr (RES) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] += __bfloat162float(*at(rblk(i), j));
+        for (int j = 0; j < 32; ++j) v[j] = __fadd_rn(v[j], __bfloat162float(*at(rblk(i), j)));
       }
 #pragma unroll
       for (int j = 0; j < 32; ++j) {

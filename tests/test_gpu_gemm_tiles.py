@@ -141,3 +141,22 @@ def test_gemm_single_tile_history_only(cuda, M, N, K, rpb, gated):
     assert rel_l2(f64(buf[0, :M]), y) < 4e-3
     assert rel_l2(f64(buf[1, :M]), f64(buf[0, :M]) - f64(base)) < 4e-3
     assert torch.all(buf[:, M] == 5.0)
+
+
+# The same product in a normal and in a swapped tile: the gate's product is rounded
+# before the residual is added in both, so the outputs are the same bits.  (Added in
+# one rounding, about 6 of a million stored values differ: 40 draws of 32640.)
+@pytest.mark.gpu
+def test_gemm_single_tile_same_bits(cuda):
+    M, K = 255, 640                                     # below 256 rows: single CTAs; 256 columns normal, 128 swapped
+    for seed in range(40):
+        a, w, bias = randn((M, K), "bf16", 5 * seed), randn((128, K), "bf16", 5 * seed + 1, 0.05), randn(128, "bf16", 3)
+        gate, resid, outs = randn((1, 128), "f32", 5 * seed + 2), randn((M, 128), "bf16", 5 * seed + 3), []
+        for n in (1, 2):
+            r = resid.repeat(1, n)
+            out, hist = torch.empty_like(r), torch.empty_like(r)
+            ff.featfix_op_gemm("bf16", a, w.repeat(n, 1), out, bias=bias.repeat(n), gate=gate.repeat(1, n),
+                               gate_stride=128 * n, rows_per_batch=M, resid=r, hist_base=r, hist_out=hist)
+            torch.cuda.synchronize()
+            outs.append((out[:, :128], hist[:, :128]))
+        assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
