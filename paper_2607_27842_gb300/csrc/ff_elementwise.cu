@@ -1,6 +1,7 @@
 // Bandwidth-bound kernels of the FeatFix denoising step: the draft (Eq. 2),
 // the fused paid check / forward (Eqs. 3-5), adaLN LayerNorm-modulation,
 // conditioning tables, embedding, sampler update and the seeded latent.
+// (Times in the comments: launches back to back in a CUDA graph.)
 #include "ff_common.cuh"
 
 #include <cooperative_groups.h>
